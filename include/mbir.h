@@ -118,7 +118,13 @@ mbir_status mbir_backproject(mbir_plan *plan, const float *s, float *x, int n_ma
  * more for finer bins); the sums are exact integer sums, so the result is
  * bitwise reproducible.  A non-finite input makes its channel's image NaN.
  * It needs 8 bytes x n_mat_max x n_pix of plan scratch.  3-D (cone): 0 =
- * tile scatter (default): a CTA per 8 x 8 x 16-voxel tile runs over every
+ * voxel-driven over detector columns (default: the in-plane weights and the
+ * row spacing of a column are common to its rays; FP32 sums over at most 32
+ * views, added in a fixed order, so bitwise reproducible; a non-finite input
+ * makes its channel's image NaN).  Plans with rays that the z axis drives, with
+ * more than 48 detector rows per voxel layer's reach or with the source within
+ * four voxels of the volume's radius run a tile scatter instead: a CTA per
+ * 8 x 8 x 16-voxel tile runs over every
  * view, stages the rays of the tile's detector box and adds each (ray, tile
  * plane) sample's bilinear terms to 32-bit fixed-point shared-memory
  * accumulators, flushed into exact 64-bit sums every vb views; each term is
@@ -148,11 +154,9 @@ mbir_status mbir_plan_set_tiling(mbir_plan *plan, int views_per_cta);
  * 90/120/180 views per CTA (written to *views_per_cta if non-NULL), then the
  * forward projection of n_channels / 2 (at least 1) basis images by one
  * thread per ray and by the strip kernel with 32/64/128/256 bins (and
- * 256 / that many views) per CTA.  Cone-beam plans: the tile scatter (where
- * available; 16- and 8-voxel-deep tiles), the direct voxel gather and the
- * split-table gather, then the
- * forward's per-lane and warp-aligned marches (mbir_plan_set_projector modes
- * 1 and 2; equal results).  Synchronises; allocates and
+ * 256 / that many views) per CTA.  Cone-beam plans: mode 0 (the tile
+ * scatter with 16- and 8-voxel-deep tiles where mode 0 is that), the direct
+ * voxel gather and the split-table gather.  Synchronises; allocates and
  * frees temporary device buffers; not allowed while `stream` is capturing
  * (MBIR_ERR_ARG).  MBIR_ERR_ARG if n_channels is outside 1..n_mat_max; on
  * any error the plan keeps its previous choices. */
@@ -160,7 +164,8 @@ mbir_status mbir_plan_autotune(mbir_plan *plan, int n_channels, mbir_stream stre
 /* Bins per CTA of the strip forward (mode 2): 32, 64, 128 or 256, with
  * 256 / bins views per CTA; MBIR_ERR_ARG otherwise.  Work split only. */
 mbir_status mbir_plan_set_strip_bins(mbir_plan *plan, int bins);
-/* Depth of the cone tile transpose's tiles (mode 0): 8 x 8 x 16 voxels
+/* Depth of the cone tile transpose's tiles (mode 0, plans that the column
+ * transpose does not cover; otherwise without effect): 8 x 8 x 16 voxels
  * (default; 256 threads, four voxels each) or 8 x 8 x 8 (two voxels per
  * thread, five CTAs per SM).  Work split only: both give the same terms and
  * the same fixed-point grid.  MBIR_ERR_ARG for a 2-D plan or another depth. */
@@ -176,9 +181,9 @@ mbir_status mbir_plan_tuning(const mbir_plan *plan, int *fwd_mode, int *strip_bi
  * from L1/L2, eight samples summed before each compensated add
  * (deterministic); 2 = rays of a block of views and bins march
  * shared-memory strips of the image, every lane on the same driving index
- * (deterministic).  Cone beam: one thread per ray; 1 (and 0) = each lane
- * marches its own range, 2 = the lanes of a warp march the same plane index
- * (same samples and sums).  All use the same per-ray Joseph weights.
+ * (deterministic).  Cone beam: one algorithm whatever the mode (a warp per
+ * detector column, lanes on its rows; one thread per ray for plans with rays
+ * that the z axis drives).  All use the same per-ray Joseph weights.
  * MBIR_ERR_ARG for other modes. */
 mbir_status mbir_plan_set_projector(mbir_plan *plan, int mode);
 
@@ -242,7 +247,7 @@ mbir_status mbmd_objective(mbir_plan *plan, const mbmd_spectrum *spec, const flo
  * A^T of the per-ray derivative, recomputing l = A x and exp(-Q l) instead of
  * storing them) or l (plan == NULL).  grad has the shape of x_or_l
  * (overwritten); objective (device, nullable) receives L.  On a cone plan
- * whose transpose is the tile scatter, every gradient channel keeps its
+ * whose transpose is the fixed-point tile scatter, every gradient channel keeps its
  * terms to 2^-12 of the fixed-point unit (the low words of
  * mbir_plan_set_backprojector's mode 0). */
 mbir_status mbmd_gradient(mbir_plan *plan, const mbmd_spectrum *spec, const float *x_or_l, const float *y,
@@ -419,7 +424,7 @@ mbir_status psps_state_destroy(psps_state *st);
  * PSPS_FLAG_LINESEARCH) and the update x += alpha p.  If objective_history
  * (HOST, length n_iter + 1) is non-NULL the call synchronises and writes
  * Phi before each iteration and after the last one (after an exact
- * re-projection).  On a cone plan whose transpose is the tile scatter, the
+ * re-projection).  On a cone plan whose transpose is the fixed-point tile scatter, the
  * cross-material Fourier and wavelet preconditioners (which difference the
  * materials' gradient numerators after a spatial filter) get the gradient
  * channels to 2^-12 of the fixed-point unit (low words), the other kinds

@@ -78,8 +78,8 @@ class Plan:
         self.sino_shape = tuple(geom.sino_shape)
 
     def set_backprojector(self, mode: str):
-        """'tile' (default: fixed-point tile scatter, deterministic), 'gather'
-        (pixel / voxel gather, FP32, deterministic), 'atomic' (ray-driven
+        """'tile' (default: 2-D fixed-point tile scatter, cone detector
+        columns; deterministic), 'gather' (pixel / voxel gather, FP32, deterministic), 'atomic' (ray-driven
         scatter with global atomics) or, for cone plans, 'split' (the voxel
         gather with split tables, bitwise equal to 'gather')."""
         _call(lib().mbir_plan_set_backprojector, self.h, {"tile": 0, "gather": 1, "atomic": 2, "split": 3}[mode])
@@ -109,14 +109,14 @@ class Plan:
 
     def set_cone_tile(self, depth: int):
         """Depth (16 or 8 voxels) of the cone tile transpose's 8 x 8 x depth
-        tiles (cone plans only)."""
+        tiles (cone plans only; plans that the column transpose covers do
+        not use it)."""
         _call(lib().mbir_plan_set_cone_tile, self.h, int(depth))
 
     def set_projector(self, mode: str):
         """2-D: 'ray' (one thread per ray), 'strip' (shared-memory strips) or
-        'tile'; cone beam: 'ray' (each lane marches its own range) or
-        'aligned' (the lanes of a warp march together; the same mode number
-        as 'strip')."""
+        'tile'; cone beam: one algorithm whatever the mode ('aligned' is the
+        mode number of 'strip')."""
         _call(lib().mbir_plan_set_projector, self.h, {"tile": 0, "ray": 1, "strip": 2, "aligned": 2}[mode])
 
     def __del__(self):

@@ -217,16 +217,16 @@ struct mbir_plan {
     psps::DBuf<float4> ray;       // (f0, df, w, bits(axis,lo,hi))
     // 2-D per-view constants for the pixel-driven transpose
     psps::DBuf<float4> view;      // parallel: (cos, sin, -, -); fan: (sx, sy, beta + pi, -)
-    int back_mode = 0;            // 0 tile scatter (default), 1 pixel / voxel gather, 2 ray-driven atomics, 3 split-table gather (3-D)
+    int back_mode = 0;            // 0 default (2-D tile scatter; 3-D columns or tile scatter), 1 pixel / voxel gather, 2 ray-driven atomics, 3 split-table gather (3-D)
     int back_views = 60;          // views per CTA of the tile transpose
     int fwd_mode = 1;             // 0 tile sums, 1 one thread per ray (default), 2 shared-memory strips
     int strip_bins = 64;          // strip forward: bins per CTA (32, 64, 128 or 256; 256 / it views)
-    // 3-D per-ray Joseph set-up (cone_ray, computed once): (fb_mid, dfb,
+    // 3-D per-ray Joseph set-up (cone_ray, computed once; general kernels): (fb_mid, dfb,
     // fc_mid, dfc) in `ray` and (weight, bits(axis | lo << 2 | hi << 17)) in
     // ray3b; per view, the set of driving axes its rays use (bit a)
     psps::DBuf<float2> ray3b;
     psps::DBuf<int> view_axes;
-    psps::DBuf<float> wsino;      // 3-D gather: weighted sinogram, up to 4 channels interleaved
+    psps::DBuf<float> wsino;      // 3-D transposes: weighted sinogram, up to 4 channels interleaved
     // scratch: packed / transposed image copies for the forward projector
     // (3-D: one copy per driving axis)
     psps::DBuf<float> xrow, xcol, xcol3;
@@ -248,6 +248,16 @@ struct mbir_plan {
     int tile_fine = 0;
     // 3-D tile transpose: tile depth (16 or 8 voxels; 8 x 8 across)
     int cone_tile = 16;
+    // 3-D detector columns (cone_cols.cuh): constants per (view, column);
+    // whether no ray is z-driven (the column forward applies) and the rows the
+    // column transpose takes per column (0: it does not apply), its split of
+    // the views and their partial images
+    psps::DBuf<float4> col;
+    psps::DBuf<float2> colw;
+    psps::DBuf<int> view_cols;    // per view, the driving axes of its columns (bit a)
+    bool cols = false;
+    int col_rows = 0, col_splits = 1, col_vchunk = 0;
+    psps::DBuf<float> col_part;
 };
 
 struct mbmd_spectrum {

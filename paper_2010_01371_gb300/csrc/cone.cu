@@ -6,39 +6,40 @@
 // b, c (b = y for x-driven rays, else x; c = y for z-driven rays, else z),
 // zero outside the volume, weight delta_a |d| / |d_a|.
 //
-// Per-ray set-up in FP32 without cancellation: the crossing of the ray with
-// the central plane of its driving axis is written in closed form from the
-// source-detector geometry (for an x-driven ray y0 = -sid u / d_x and
-// z0 = -sid cos(beta) w / d_x, with u, w the detector offsets), so the
-// interpolation coordinates f(i) = f_mid + (i - c_a) df carry no
-// large-number rounding.
+// The detector rows run along z, so every ray of one detector column (a view
+// and a column index) takes the same in-plane path: its driving axis a (x or
+// y) and its coordinate b(i) = b0 + (i - c_a) db do not depend on the row, and
+// on plane i its height is z = (row offset) k(i) with k(i) = q0 + (i - c_a) dq
+// common to the column.  These four numbers per column are set up in FP64 once
+// per plan (cone_cols.cuh); cone_cols.cu holds the forward and the transpose
+// built on them, which every plan without z-driven rays uses.
 //
-// The set-up runs once per plan and is stored per ray (24 bytes: 1.7 GB for
-// 360 x 384 x 512 rays; the central-plane coordinates less 1/2, for the
-// conversion-free sample split), so the forward and the transposes read
-// bitwise the same interpolation coordinates and weights.
+// This file holds the set-up and the general kernels: plans with z-driven rays
+// (detector half-height above sdd / sqrt 2) and the alternative transposes.
+// They read a per-ray table (24 bytes per ray) derived from the column
+// constants: coordinates relative to the middle of the volume (index n / 2
+// of the interpolated axis, less 1/2 for the conversion-free sample split),
+// so that FP32 spends no bits on the offset.
 //
-// Forward: one thread per ray (neighbouring threads = neighbouring detector
-// columns of one row), reading a packed copy of the volume laid out so the
-// two interpolated axes are the fastest (b fastest), for each driving axis;
-// Kahan-compensated FP32 sums.
-//
-// Transpose (default): voxel-driven gather, one thread per voxel, no atomics
-// (bitwise reproducible), reading a weighted copy of the sinogram with up to
-// four channels interleaved per ray (16 bytes per ray of plan scratch).  For every view and every driving axis a that the
-// view's rays use, the voxel's bilinear footprint on the plane of its own
-// driving index (the voxel centre +- one voxel in the two interpolated axes)
-// is projected onto the detector; every detector cell whose centre lies in the
-// bounding box of the projected corners is a candidate ray, and a candidate
-// contributes exactly the forward's weight of this voxel: its driving axis
-// must be a and the ray's sample split must put the voxel on one of its four
-// taps.  The ray-driven scatter with global FP32 atomics
-// remains as the alternative (mbir_plan_set_backprojector mode 2).
+// Transposes here: a ray-driven tile scatter with fixed-point sums (mode 0 of
+// plans that the column kernels do not cover), voxel-driven gathers (modes 1
+// and 3) and a ray-driven scatter with global FP32 atomics (mode 2).  The
+// gathers: one thread per voxel, no atomics (bitwise reproducible), reading a
+// weighted copy of the sinogram with up to four channels interleaved per ray
+// (16 bytes per ray of plan scratch).  For every view and every driving axis a
+// that the view's rays use, the voxel's bilinear footprint on the plane of its
+// own driving index (the voxel centre +- one voxel in the two interpolated
+// axes) is projected onto the detector; every detector cell whose centre lies
+// in the bounding box of the projected corners is a candidate ray, and a
+// candidate contributes exactly the forward's weight of this voxel: its
+// driving axis must be a and the ray's sample split must put the voxel on one
+// of its four taps.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
+#include "cone_cols.cuh"
 
 namespace psps {
 namespace {
@@ -74,55 +75,43 @@ __device__ __forceinline__ void range_1d(float f_mid, float df, float ca, int n_
     hi = fminf(t1, 1.0e8f);
 }
 
-__device__ __forceinline__ ConeRay cone_ray(const mbir_geometry &g, float4 V, int iu, int iv) {
-    // V = (sx, sy, cos beta, sin beta)
-    const float u = (float)((iu - 0.5 * (g.n_u - 1)) * g.du), w = (float)((iv - 0.5 * (g.n_v - 1)) * g.dv);
-    const float sdd = (float)g.sdd, sid = (float)g.sid;
-    const float d0 = -sdd * V.z - u * V.w, d1 = -sdd * V.w + u * V.z, d2 = w;
-    const float a0 = fabsf(d0), a1 = fabsf(d1), a2 = fabsf(d2);
-    const float nd = sqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+// Set-up of ray (column constants C, W of its column; row iv).  fb_mid and
+// fc_mid are relative to index n / 2 of their axes and less 1/2.
+__device__ __forceinline__ ConeRay cone_ray(const mbir_geometry &g, float4 V, float4 C, float2 W, int iu, int iv) {
     const float dx = (float)g.dx, dy = (float)g.dy, dz = (float)g.dz;
-    const float cx = 0.5f * (g.nx - 1), cy = 0.5f * (g.ny - 1), cz = 0.5f * (g.nz - 1);
+    const float row = (float)iv - 0.5f * (g.n_v - 1), w = row * (float)g.dv;
+    const float u = (float)((iu - 0.5 * (g.n_u - 1)) * g.du);
+    const float d0 = -(float)g.sdd * V.z - u * V.w, d1 = -(float)g.sdd * V.w + u * V.z, a2 = fabsf(w);
     ConeRay r;
-    if (a0 >= a1 && a0 >= a2) {
-        r.axis = 0;
-        const float y0 = -sid * u / d0, z0 = -sid * V.z * w / d0;
-        r.fb_mid = y0 / dy + cy;
-        r.dfb = dx * (d1 / d0) / dy;
-        r.fc_mid = z0 / dz + cz;
-        r.dfc = dx * (d2 / d0) / dz;
-        r.ca = cx;
-        r.w = dx * nd / a0;
-    } else if (a1 >= a2) {
-        r.axis = 1;
-        const float x0 = sid * u / d1, z0 = -sid * V.w * w / d1;
-        r.fb_mid = x0 / dx + cx;
-        r.dfb = dy * (d0 / d1) / dx;
-        r.fc_mid = z0 / dz + cz;
-        r.dfc = dy * (d2 / d1) / dz;
-        r.ca = cy;
-        r.w = dy * nd / a1;
-    } else {
-        r.axis = 2;
-        // crossing of the source plane z = 0: the source itself
-        r.fb_mid = V.x / dx + cx;
-        r.dfb = dz * (d0 / d2) / dx;
-        r.fc_mid = V.y / dy + cy;
-        r.dfc = dz * (d1 / d2) / dy;
-        r.ca = cz;   // plane z = 0 is index cz; the source sits there
-        r.w = dz * nd / a2;
-    }
-    const int na = r.axis == 0 ? g.nx : (r.axis == 1 ? g.ny : g.nz);
-    const int nb = r.axis == 0 ? g.ny : g.nx;
-    const int nc = r.axis == 2 ? g.ny : g.nz;
     float l0, h0, l1, h1;
-    range_1d(r.fb_mid, r.dfb, r.ca, nb, na, l0, h0);
-    range_1d(r.fc_mid, r.dfc, r.ca, nc, na, l1, h1);
+    int na;
+    if (a2 > fmaxf(fabsf(d0), fabsf(d1))) {
+        // z drives: the plane z = 0 holds the source, so the ray crosses it there
+        r.axis = 2;
+        r.fb_mid = V.x / dx + 0.5f * (g.nx - 1) - 0.5f - (float)(g.nx >> 1);
+        r.dfb = dz * (d0 / w) / dx;
+        r.fc_mid = V.y / dy + 0.5f * (g.ny - 1) - 0.5f - (float)(g.ny >> 1);
+        r.dfc = dz * (d1 / w) / dy;
+        r.ca = 0.5f * (g.nz - 1);
+        r.w = dz * sqrtf(d0 * d0 + d1 * d1 + w * w) / a2;
+        na = g.nz;
+        range_1d(r.fb_mid + 0.5f + (float)(g.nx >> 1), r.dfb, r.ca, g.nx, na, l0, h0);
+        range_1d(r.fc_mid + 0.5f + (float)(g.ny >> 1), r.dfc, r.ca, g.ny, na, l1, h1);
+    } else {
+        int lo, hi;
+        decode_col(W, r.axis, lo, hi);
+        r.fb_mid = C.x, r.dfb = C.y;
+        r.fc_mid = fmaf(row, C.z, cone_z_offset(g.nz));
+        r.dfc = row * C.w;
+        na = r.axis == 0 ? g.nx : g.ny;
+        r.ca = 0.5f * (na - 1);
+        r.w = cone_weight(g, W, u, w);
+        l0 = (float)lo, h0 = (float)hi;
+        range_1d(r.fc_mid + 0.5f + (float)(g.nz >> 1), r.dfc, r.ca, g.nz, na, l1, h1);
+    }
     const float lo = fmaxf(fmaxf(l0, l1), 0.f), hi = fminf(fminf(h0, h1), (float)(na - 1));
-    r.lo = (int)floorf(lo) - 1;
-    r.hi = (int)ceilf(hi) + 1;
-    if (r.lo < 0) r.lo = 0;
-    if (r.hi > na - 1) r.hi = na - 1;
+    r.lo = max((int)floorf(lo) - 1, 0);
+    r.hi = min((int)ceilf(hi) + 1, na - 1);
     return r;
 }
 
@@ -135,19 +124,56 @@ __global__ void setup_view3d_kernel(mbir_geometry g, float4 *vt) {
     vt[v] = make_float4((float)(g.sid * c), (float)(g.sid * s), (float)c, (float)s);
 }
 
-__global__ void setup_rays3d_kernel(mbir_geometry g, const float4 *__restrict__ vt, int64_t n_rays,
-                                    float4 *__restrict__ ta, float2 *__restrict__ tb, int *__restrict__ view_axes) {
-    const int64_t ray = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ray >= n_rays) return;
+// Column constants (see cone_cols.cuh) and the driving-index range in which
+// the column's in-plane coordinate lies in (-1, n), widened by one index.
+__global__ void setup_cols3d_kernel(mbir_geometry g, float4 *__restrict__ col, float2 *__restrict__ colw,
+                                    int *__restrict__ view_cols) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= (int64_t)g.n_views * g.n_u) return;
+    const int v = (int)(j / g.n_u), iu = (int)(j % g.n_u);
+    double s, c;
+    sincos(g.angle0 + v * (g.angle_span / g.n_views), &s, &c);
+    const double u = (iu - 0.5 * (g.n_u - 1)) * g.du;
+    const double d0 = -g.sdd * c - u * s, d1 = -g.sdd * s + u * c;
+    const bool xd = fabs(d0) >= fabs(d1);
+    const double da = xd ? d0 : d1, db = xd ? d1 : d0, ha = xd ? g.dx : g.dy, hb = xd ? g.dy : g.dx;
+    const int na = xd ? g.nx : g.ny, nb = xd ? g.ny : g.nx;
+    // crossing of the central plane of the driving axis, in closed form
+    const double b0 = (xd ? -1.0 : 1.0) * g.sid * u / da / hb + 0.5 * (nb - 1);
+    const double slope = ha * (db / da) / hb;
+    const double q0 = -g.sid * (xd ? c : s) / da * g.dv / g.dz, dq = ha / da * g.dv / g.dz;
+    double lo = 0.0, hi = na - 1.0;
+    if (slope != 0.0) {
+        const double ta = (-1.0 - b0) / slope + 0.5 * (na - 1), tb = (nb - b0) / slope + 0.5 * (na - 1);
+        lo = fmax(lo, floor(fmin(ta, tb)) - 1.0);
+        hi = fmin(hi, ceil(fmax(ta, tb)) + 1.0);
+    } else if (!(b0 > -1.0 && b0 < nb)) {
+        hi = -1.0;
+    }
+    if (lo > hi) lo = 1.0, hi = 0.0;
+    col[j] = make_float4((float)(b0 - 0.5 - (nb >> 1)), (float)slope, (float)q0, (float)dq);
+    colw[j] = make_float2((float)(ha / fabs(da)), __int_as_float((xd ? 0 : 1) | ((int)lo << 2) | ((int)hi << 17)));
+    atomicOr(view_cols + v, xd ? 1 : 2);
+}
+
+// One view per blockIdx.y.  A view's axis bits are set by the first rays that
+// have them (a plain read first: one atomic per ray on a few words took most
+// of a plan's set-up, 34 ms at 360 x 384 x 512 rays).
+__global__ void setup_rays3d_kernel(mbir_geometry g, const float4 *__restrict__ vt, const float4 *__restrict__ col,
+                                    const float2 *__restrict__ colw, float4 *__restrict__ ta, float2 *__restrict__ tb,
+                                    int *view_axes) {
     const int per_view = g.n_u * g.n_v;
-    const int v = (int)(ray / per_view);
-    const int rem = (int)(ray % per_view);
-    const ConeRay r = cone_ray(g, vt[v], rem % g.n_u, rem / g.n_u);
-    ta[ray] = make_float4(r.fb_mid - 0.5f, r.dfb, r.fc_mid - 0.5f, r.dfc);
-    const bool empty = r.lo > r.hi;
-    const int bits = r.axis | ((empty ? 1 : r.lo) << 2) | ((empty ? 0 : r.hi) << 17);
-    tb[ray] = make_float2(r.w, __int_as_float(bits));
-    if (!empty) atomicOr(view_axes + v, 1 << r.axis);
+    for (int v = blockIdx.y; v < g.n_views; v += gridDim.y)
+        for (int rem = blockIdx.x * blockDim.x + threadIdx.x; rem < per_view; rem += gridDim.x * blockDim.x) {
+            const int iv = rem / g.n_u, iu = rem - iv * g.n_u;
+            const int64_t ray = (int64_t)v * per_view + rem, cj = (int64_t)v * g.n_u + iu;
+            const ConeRay r = cone_ray(g, vt[v], col[cj], colw[cj], iu, iv);
+            ta[ray] = make_float4(r.fb_mid, r.dfb, r.fc_mid, r.dfc);
+            const bool empty = r.lo > r.hi;
+            const int bits = r.axis | ((empty ? 1 : r.lo) << 2) | ((empty ? 0 : r.hi) << 17);
+            tb[ray] = make_float2(r.w, __int_as_float(bits));
+            if (!empty && !((*(volatile int *)(view_axes + v) >> r.axis) & 1)) atomicOr(view_axes + v, 1 << r.axis);
+        }
 }
 
 __device__ __forceinline__ void decode3(float2 b, int &axis, int &lo, int &hi) {
@@ -157,204 +183,68 @@ __device__ __forceinline__ void decode3(float2 b, int &axis, int &lo, int &hi) {
     hi = (bits >> 17) & 0x7fff;
 }
 
-// Packed copies of x[m][z][y][x] for the three driving axes, materials
-// innermost with stride P: layout[a][c][b][m] (see the file comment), each
-// plane of the driving axis with kPad zero cells on both sides of b and c,
-// so that every tap of every sample a ray's range can take lies inside the
-// copy and reads the value or a zero (no bounds tests in the forward).
-constexpr int kPad = 2;
-
-__host__ __device__ inline int64_t pack3d_floats(int nx, int ny, int nz) {
-    const int64_t a = (int64_t)nx * (nz + 2 * kPad) * (ny + 2 * kPad);   // a = x: [ix][iz][iy]
-    const int64_t b = (int64_t)ny * (nz + 2 * kPad) * (nx + 2 * kPad);   // a = y: [iy][iz][ix]
-    const int64_t c = (int64_t)nz * (ny + 2 * kPad) * (nx + 2 * kPad);   // a = z: [iz][iy][ix]
-    return 4 * (a > b ? (a > c ? a : c) : (b > c ? b : c));
-}
-
-// Zero the kPad-wide borders of the three packed copies (the interiors are
-// written by pack3d_kernel), P floats per cell.
-__global__ void pack3d_border_kernel(int P, int nx, int ny, int nz, float *__restrict__ ox, float *__restrict__ oy,
-                                     float *__restrict__ oz) {
-    const int W = 2 * kPad;
-    for (int a = 0; a < 3; ++a) {
-        const int na = a == 0 ? nx : (a == 1 ? ny : nz);
-        const int nb = a == 0 ? ny : nx, nc = a == 2 ? ny : nz;
-        const int64_t plane = (int64_t)(nc + W) * (nb + W);
-        float *o = a == 0 ? ox : (a == 1 ? oy : oz);
-        const int64_t n = (int64_t)na * plane;
-        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-            const int rem = (int)(k % plane);
-            const int c = rem / (nb + W), b = rem % (nb + W);
-            if (c >= kPad && c < nc + kPad && b >= kPad && b < nb + kPad) continue;
-            for (int m = 0; m < P; ++m) o[k * P + m] = 0.f;
-        }
-    }
-}
-
-__global__ void pack3d_kernel(const float *__restrict__ x, int nm, int P, int nx, int ny, int nz,
-                              float *__restrict__ ox, float *__restrict__ oy, float *__restrict__ oz) {
-    const int64_t n = (int64_t)nx * ny * nz;
-    const int W = 2 * kPad;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(j % nx);
-        const int iy = (int)((j / nx) % ny);
-        const int iz = (int)(j / ((int64_t)nx * ny));
-        const int64_t px = (((int64_t)ix * (nz + W) + iz + kPad) * (ny + W) + iy + kPad) * P;   // [ix][iz][iy]
-        const int64_t py = (((int64_t)iy * (nz + W) + iz + kPad) * (nx + W) + ix + kPad) * P;   // [iy][iz][ix]
-        const int64_t pz = (((int64_t)iz * (ny + W) + iy + kPad) * (nx + W) + ix + kPad) * P;   // [iz][iy][ix]
-        for (int m = 0; m < P; ++m) {
-            const float v = m < nm ? x[m * n + j] : 0.f;
-            ox[px + m] = v;
-            oy[py + m] = v;
-            oz[pz + m] = v;
-        }
-    }
-}
-
+// One thread per ray, each over its own range; two samples' tap loads are
+// issued before use.  Copies of the volume as cone_cols.cuh describes; a
+// sample's lower tap indices are clamped to [-kPad, n + kPad - 2]: a sample the
+// clamp moves lies wholly outside the volume (its taps are at <= -2 or >= n),
+// and the clamped taps then read border zeros, as the true ones are.
 template <int NM>
-struct P3;
-template <>
-struct P3<1> {
-    using T = float;
-    __device__ static void get(const T &v, float (&o)[1]) { o[0] = v; }
-};
-template <>
-struct P3<2> {
-    using T = float2;
-    __device__ static void get(const T &v, float (&o)[2]) {
-        o[0] = v.x;
-        o[1] = v.y;
-    }
-};
-template <>
-struct P3<4> {
-    using T = float4;
-    __device__ static void get(const T &v, float (&o)[4]) {
-        o[0] = v.x;
-        o[1] = v.y;
-        o[2] = v.z;
-        o[3] = v.w;
-    }
-};
-
-// ALIGNED: the lanes of a warp (neighbouring detector columns of one row)
-// step the same driving index over the union of their ranges, each adding
-// only inside its own range, so that one load instruction of the warp reads
-// neighbouring voxels of one plane (a few cache lines) instead of one plane
-// per lane.  Same samples, weights and summation order either way.
-template <int NM, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads)
     fwd_cone_kernel(mbir_geometry g, const float4 *__restrict__ ta, const float2 *__restrict__ tb,
-                    const typename P3<NM>::T *__restrict__ ox, const typename P3<NM>::T *__restrict__ oy,
-                    const typename P3<NM>::T *__restrict__ oz, int nm, int64_t n_rays, float *__restrict__ l) {
+                    const typename CPack<NM>::T *__restrict__ ox, const typename CPack<NM>::T *__restrict__ oy,
+                    const typename CPack<NM>::T *__restrict__ oz, int nm, int64_t n_rays, float *__restrict__ l) {
     const int64_t ray = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (ALIGNED) {
-        if (((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) >= n_rays) return;   // whole warp past the end
-    } else if (ray >= n_rays) {
-        return;
-    }
-    const bool live = ray < n_rays;
-    const float4 A = live ? ta[ray] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float2 B = live ? tb[ray] : make_float2(0.f, __int_as_float(1 << 2));   // empty range lo 1 > hi 0
+    if (ray >= n_rays) return;
+    const float4 A = ta[ray];
+    const float2 B = tb[ray];
     int axis, lo, hi;
     decode3(B, axis, lo, hi);
-    int i_lo = lo, i_hi = hi;
-    if (ALIGNED) {
-        // rays that miss the volume (lo > hi) do not widen the warp's range
-        if (lo > hi) i_lo = 0x7fffffff, i_hi = -1;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            i_lo = min(i_lo, __shfl_xor_sync(0xffffffffu, i_lo, o));
-            i_hi = max(i_hi, __shfl_xor_sync(0xffffffffu, i_hi, o));
-        }
-    }
-    const typename P3<NM>::T *src = axis == 0 ? ox : (axis == 1 ? oy : oz);
-    // padded plane: (nc + 2 kPad) rows of (nb + 2 kPad) cells.  A sample's
-    // lower tap indices are clamped to [-kPad, n + kPad - 2]: a sample the
-    // clamp moves lies wholly outside the volume (its taps are at <= -2 or
-    // >= n), and the clamped taps then read border zeros, as the true ones
-    // are; every other sample reads its own taps.
+    using T = typename CPack<NM>::T;
+    const T *src = axis == 0 ? ox : (axis == 1 ? oy : oz);
     const int nb = axis == 0 ? g.ny : g.nx, nc = axis == 2 ? g.ny : g.nz;
-    const int nbp = nb + 2 * kPad, ncp = nc + 2 * kPad;
+    const int nbp = nb + 2 * kPad, ncp = nc + 2 * kPad, cb = nb >> 1, cc = nc >> 1;
     const float ca = 0.5f * ((axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nz)) - 1);
     float acc[NM], comp[NM];
 #pragma unroll
     for (int m = 0; m < NM; ++m) acc[m] = comp[m] = 0.f;
-    int i = i_lo;
-    if (!ALIGNED) {
-        // Two samples per step: their eight tap loads (addresses clamped into
-        // the volume, values zeroed outside it) are issued before use; the
-        // taps and samples are then added in the one-at-a-time order.
-        using T = typename P3<NM>::T;
-        for (; i + 1 <= i_hi; i += 2) {
-            T v[2][4];
-            float gb[2], gc[2];
+    for (int i = lo; i <= hi; i += 2) {
+        T v[2][4];
+        float gb[2], gc[2];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const float t = (float)(i + u) - ca;
-                const int ib0 = joseph_split(fmaf(t, A.y, A.x), gb[u]), ic0 = joseph_split(fmaf(t, A.w, A.z), gc[u]);
-                const int ibc = min(max(ib0, -kPad), nb + kPad - 2), icc = min(max(ic0, -kPad), nc + kPad - 2);
-                const T *tap = src + ((int64_t)(i + u) * ncp + icc + kPad) * nbp + ibc + kPad;
-                v[u][0] = __ldg(tap);
-                v[u][1] = __ldg(tap + 1);
-                v[u][2] = __ldg(tap + nbp);
-                v[u][3] = __ldg(tap + nbp + 1);
-            }
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                float sm[NM];
-#pragma unroll
-                for (int m = 0; m < NM; ++m) sm[m] = 0.f;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float wc = (q >> 1) ? gc[u] : 1.f - gc[u];
-                    const float wbc = ((q & 1) ? gb[u] : 1.f - gb[u]) * wc;
-                    float val[NM];
-                    P3<NM>::get(v[u][q], val);
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) sm[m] = fmaf(wbc, val[m], sm[m]);
-                }
-#pragma unroll
-                for (int m = 0; m < NM; ++m) {
-                    const float yk = __fsub_rn(sm[m], comp[m]);
-                    const float tt = __fadd_rn(acc[m], yk);
-                    comp[m] = __fsub_rn(__fsub_rn(tt, acc[m]), yk);
-                    acc[m] = tt;
-                }
-            }
+        for (int u = 0; u < 2; ++u) {
+            const int iu = min(i + u, hi);
+            const float t = (float)iu - ca;
+            const int ib0 = joseph_split(fmaf(t, A.y, A.x), gb[u]) + cb, ic0 = joseph_split(fmaf(t, A.w, A.z), gc[u]) + cc;
+            const int ibc = min(max(ib0, -kPad), nb + kPad - 2), icc = min(max(ic0, -kPad), nc + kPad - 2);
+            const T *tap = src + ((int64_t)iu * nbp + ibc + kPad) * ncp + icc + kPad;
+            v[u][0] = __ldg(tap);
+            v[u][1] = __ldg(tap + 1);
+            v[u][2] = __ldg(tap + ncp);
+            v[u][3] = __ldg(tap + ncp + 1);
         }
-    }
-    for (; i <= i_hi; ++i) {
-        if (ALIGNED && (i < lo || i > hi)) continue;
-        const float t = (float)i - ca;
-        float gb, gc;
-        const int ib0 = joseph_split(fmaf(t, A.y, A.x), gb), ic0 = joseph_split(fmaf(t, A.w, A.z), gc);
-        float s[NM];
 #pragma unroll
-        for (int m = 0; m < NM; ++m) s[m] = 0.f;
-        const int ibc = min(max(ib0, -kPad), nb + kPad - 2), icc = min(max(ic0, -kPad), nc + kPad - 2);
-        const typename P3<NM>::T *tap = src + ((int64_t)i * ncp + icc + kPad) * nbp + ibc + kPad;
+        for (int u = 0; u < 2; ++u) {
+            if (i + u > hi) break;
+            float sm[NM];
 #pragma unroll
-        for (int jc = 0; jc < 2; ++jc) {
-            const float wc = jc ? gc : 1.f - gc;
+            for (int m = 0; m < NM; ++m) sm[m] = 0.f;
 #pragma unroll
-            for (int jb = 0; jb < 2; ++jb) {
-                const float wbc = (jb ? gb : 1.f - gb) * wc;
+            for (int q = 0; q < 4; ++q) {
+                const float wbc = ((q >> 1) ? gb[u] : 1.f - gb[u]) * ((q & 1) ? gc[u] : 1.f - gc[u]);
                 float val[NM];
-                P3<NM>::get(__ldg(tap + jc * nbp + jb), val);
+                CPack<NM>::get(v[u][q], val);
 #pragma unroll
-                for (int m = 0; m < NM; ++m) s[m] = fmaf(wbc, val[m], s[m]);
+                for (int m = 0; m < NM; ++m) sm[m] = fmaf(wbc, val[m], sm[m]);
+            }
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                const float yk = __fsub_rn(sm[m], comp[m]);
+                const float tt = __fadd_rn(acc[m], yk);
+                comp[m] = __fsub_rn(__fsub_rn(tt, acc[m]), yk);
+                acc[m] = tt;
             }
         }
-#pragma unroll
-        for (int m = 0; m < NM; ++m) {
-            const float yk = __fsub_rn(s[m], comp[m]);
-            const float tt = __fadd_rn(acc[m], yk);
-            comp[m] = __fsub_rn(__fsub_rn(tt, acc[m]), yk);
-            acc[m] = tt;
-        }
     }
-    if (!live) return;
 #pragma unroll
     for (int m = 0; m < NM; ++m)
         if (m < nm) l[(int64_t)m * n_rays + ray] = acc[m] * B.x;
@@ -386,7 +276,8 @@ __global__ void __launch_bounds__(kThreads)
         for (int i = r.lo; i <= r.hi; ++i) {
             const float t = (float)i - r.ca;
             float gb, gc;
-            const int ib0 = joseph_split(fmaf(t, r.dfb, r.fb_mid), gb), ic0 = joseph_split(fmaf(t, r.dfc, r.fc_mid), gc);
+            const int ib0 = joseph_split(fmaf(t, r.dfb, r.fb_mid), gb) + (nb >> 1);
+            const int ic0 = joseph_split(fmaf(t, r.dfc, r.fc_mid), gc) + (nc >> 1);
             for (int jc = 0; jc < 2; ++jc) {
                 const int ic = ic0 + jc;
                 if (ic < 0 || ic >= nc) continue;
@@ -518,7 +409,8 @@ __device__ __forceinline__ void gather_cells(const mbir_geometry &g, int v, int 
                                              const float4 *s_ta, const typename Vec<C>::T *s_ws, const int *s_ax,
                                              int su0, int sv0, int sw, float (&sv)[C]) {
     const int id = A == 0 ? ix : (A == 1 ? iy : iz);                   // driving index
-    const int ib = A == 0 ? iy : ix, ic = A == 2 ? iy : iz;            // interpolated indices
+    // interpolated indices, relative to the middles that the table's coordinates refer to
+    const int ib = (A == 0 ? iy : ix) - ((A == 0 ? g.ny : g.nx) >> 1), ic = (A == 2 ? iy : iz) - ((A == 2 ? g.ny : g.nz) >> 1);
     const float t = (float)id - 0.5f * ((A == 0 ? g.nx : (A == 1 ? g.ny : g.nz)) - 1);
     const int64_t view0 = (int64_t)v * g.n_u * g.n_v;
     for (int jv = iv0; jv <= iv1; ++jv) {
@@ -709,7 +601,7 @@ __device__ __forceinline__ bool tile_box_warp(const mbir_geometry &g, const floa
     return true;
 }
 
-// Voxel-driven exact transpose with split tables (default).  Same tiles,
+// Voxel-driven exact transpose with split tables.  Same tiles,
 // candidate boxes and staging as back_cone_gather_kernel, but the staging
 // also evaluates, for every staged detector cell and each of the tile's
 // kPlanes driving planes (x- or y-driven rays), the ray's Joseph split on
@@ -796,8 +688,8 @@ __global__ void __launch_bounds__(kGX * kGY * kGZ, 4)
                     for (int q = 0; q < kPlanes; ++q) {
                         const float t = (float)(pbase + q) - ca;
                         float gb, gc;
-                        const int ib0 = joseph_split(fmaf(t, R.y, R.x), gb);
-                        const int ic0 = joseph_split(fmaf(t, R.w, R.z), gc);
+                        const int ib0 = joseph_split(fmaf(t, R.y, R.x), gb) + (nb >> 1);
+                        const int ic0 = joseph_split(fmaf(t, R.w, R.z), gc) + (g.nz >> 1);
                         const bool ok = same && ib0 >= -1 && ib0 < nb && ic0 >= -1 && ic0 < g.nz;
                         s_ij[q][k] = ok ? (unsigned)(ib0 + 1) | ((unsigned)(ic0 + 1) << 16) : kNoCell;
                         s_f[q][k] = make_float2(gb, gc);
@@ -857,8 +749,8 @@ __global__ void __launch_bounds__(kGX * kGY * kGZ, 4)
     }
 }
 
-// Ray-driven tile transpose with fixed-point shared-memory sums (mode 0,
-// the default).  A CTA owns a tile of 8 x 8 x TZ voxels (TZ = 16 or 8, chosen
+// Ray-driven tile transpose with fixed-point shared-memory sums (mode 0 of
+// the plans that the column transpose does not cover).  A CTA owns a tile of 8 x 8 x TZ voxels (TZ = 16 or 8, chosen
 // per plan) and runs over
 // every view.  For each view and each driving axis a of its rays it stages,
 // in chunks, the detector box that covers the tile's footprint (the gather's
@@ -948,8 +840,9 @@ __device__ __forceinline__ void tile3_tap(unsigned addr, float w, const float (&
 
 // The pairs (staged ray k < m, tile plane p) of driving axis A: the sample's
 // split on plane a0 + p and its terms on the taps inside the tile (b in
-// [b0, b0 + eb), c in [c0, c0 + ec); planes p < np).  NP consecutive
-// threads take the NP planes (8, or the depth for z-driven rays) of one ray.
+// [b0, b0 + eb), c in [c0, c0 + ec), relative to the axes' middles; planes
+// p < np).  NP consecutive threads take the NP planes (8, or the depth for
+// z-driven rays) of one ray.
 template <int A, int C, int NF, int TZ>
 __device__ __forceinline__ void tile3_scatter(int m, const float4 *s_ta, const typename Vec<C>::T *s_ws,
                                               const int *s_ax, int a0, int np, float ca, int b0, int eb, int c0,
@@ -1055,11 +948,14 @@ __global__ void __launch_bounds__(kTThreads, TZ == 16 ? 4 : 5)
                 }
                 __syncthreads();
                 if (A == 0)
-                    tile3_scatter<0, C, NF, TZ>(m, s_ta, s_ws, s_ax, x0, ex, cx, y0, ey, z0, ez, acc_addr);
+                    tile3_scatter<0, C, NF, TZ>(m, s_ta, s_ws, s_ax, x0, ex, cx, y0 - (g.ny >> 1), ey, z0 - (g.nz >> 1), ez,
+                                                  acc_addr);
                 else if (A == 1)
-                    tile3_scatter<1, C, NF, TZ>(m, s_ta, s_ws, s_ax, y0, ey, cy, x0, ex, z0, ez, acc_addr);
+                    tile3_scatter<1, C, NF, TZ>(m, s_ta, s_ws, s_ax, y0, ey, cy, x0 - (g.nx >> 1), ex, z0 - (g.nz >> 1), ez,
+                                                  acc_addr);
                 else
-                    tile3_scatter<2, C, NF, TZ>(m, s_ta, s_ws, s_ax, z0, ez, cz, x0, ex, y0, ey, acc_addr);
+                    tile3_scatter<2, C, NF, TZ>(m, s_ta, s_ws, s_ax, z0, ez, cz, x0 - (g.nx >> 1), ex, y0 - (g.ny >> 1), ey,
+                                                  acc_addr);
                 __syncthreads();
             }
         }
@@ -1101,7 +997,11 @@ __global__ void __launch_bounds__(kTThreads, TZ == 16 ? 4 : 5)
 
 }  // namespace
 
-int64_t cone_pack_floats(const mbir_geometry &g) { return pack3d_floats(g.nx, g.ny, g.nz); }
+int64_t cone_pack_floats(const mbir_geometry &g) {
+    const int64_t W = 2 * kPad, pz = g.nz + W, py = g.ny + W;
+    const int64_t a = g.nx * (g.ny + W) * pz, b = g.ny * (g.nx + W) * pz, c = g.nz * (g.nx + W) * py;
+    return 4 * std::max(a, std::max(b, c));
+}
 
 mbir_status cone_setup(mbir_plan *p) {
     PSPS_TRY(p->view.alloc(p->g.n_views));
@@ -1109,7 +1009,7 @@ mbir_status cone_setup(mbir_plan *p) {
     PSPS_TRY(p->ray3b.alloc(p->n_rays));
     PSPS_TRY(p->view_axes.alloc(p->g.n_views));
     PSPS_TRY(p->view_axes.zero(0));
-    PSPS_TRY(p->wsino.alloc((size_t)4 * p->n_rays));
+    PSPS_TRY(p->wsino.alloc((size_t)4 * p->g.n_views * p->g.n_u * (p->g.n_v + 2 * kRowPad)));
     PSPS_TRY(p->wmax.alloc(4));
     {
         // Rays of one view that reach one voxel j (any driving axis), for the
@@ -1140,51 +1040,44 @@ mbir_status cone_setup(mbir_plan *p) {
     }
     setup_view3d_kernel<<<(unsigned)cdiv(p->g.n_views, 128), 128>>>(p->g, p->view.p);
     PSPS_LAUNCH_CHECK();
-    setup_rays3d_kernel<<<(unsigned)cdiv(p->n_rays, kThreads), kThreads>>>(p->g, p->view.p, p->n_rays, p->ray.p,
-                                                                          p->ray3b.p, p->view_axes.p);
+    const int64_t n_cols = (int64_t)p->g.n_views * p->g.n_u;
+    PSPS_TRY(p->col.alloc(n_cols));
+    PSPS_TRY(p->colw.alloc(n_cols));
+    PSPS_TRY(p->view_cols.alloc(p->g.n_views));
+    PSPS_TRY(p->view_cols.zero(0));
+    setup_cols3d_kernel<<<(unsigned)cdiv(n_cols, kThreads), kThreads>>>(p->g, p->col.p, p->colw.p, p->view_cols.p);
     PSPS_LAUNCH_CHECK();
-    return MBIR_OK;
+    const int64_t per_view = (int64_t)p->g.n_u * p->g.n_v;
+    const dim3 grd((unsigned)std::min<int64_t>(cdiv(per_view, kThreads), 1024), (unsigned)std::min(p->g.n_views, 65535));
+    setup_rays3d_kernel<<<grd, kThreads>>>(p->g, p->view.p, p->col.p, p->colw.p, p->ray.p, p->ray3b.p, p->view_axes.p);
+    PSPS_LAUNCH_CHECK();
+    PSPS_TRY(cone_cols_setup(p));
+    // the copy of the z-driven rays, only where there are such rays
+    return p->cols ? MBIR_OK : p->xcol3.alloc(cone_pack_floats(p->g));
 }
 
 mbir_status project_cone(mbir_plan *p, const float *x, float *l, int n_mat, cudaStream_t s) {
     const mbir_geometry &g = p->g;
-    const int64_t n = p->n_pix;
     for (int m0 = 0; m0 < n_mat; m0 += 4) {
         const int nm = n_mat - m0 < 4 ? n_mat - m0 : 4;
-        const int P = nm == 1 ? 1 : (nm == 2 ? 2 : 4);
-        float *ox = p->xcol.p, *oy = p->xrow.p, *oz = p->xcol3.p;
-        const int64_t grid = cdiv(n, kThreads) < 65535 * 8 ? cdiv(n, kThreads) : 65535 * 8;
-        pack3d_border_kernel<<<1024, kThreads, 0, s>>>(P, g.nx, g.ny, g.nz, ox, oy, oz);
-        PSPS_LAUNCH_CHECK();
-        pack3d_kernel<<<(unsigned)grid, kThreads, 0, s>>>(x + m0 * n, nm, P, g.nx, g.ny, g.nz, ox, oy, oz);
-        PSPS_LAUNCH_CHECK();
-        const unsigned gr = (unsigned)cdiv(p->n_rays, kThreads);
+        const float *xm = x + (int64_t)m0 * p->n_pix;
         float *lm = l + (int64_t)m0 * p->n_rays;
-        // fwd_mode 2: warp-aligned march; otherwise each lane from its own range
-        if (p->fwd_mode == 2) {
-            if (P == 1)
-                fwd_cone_kernel<1, true><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, ox, oy, oz, nm, p->n_rays, lm);
-            else if (P == 2)
-                fwd_cone_kernel<2, true><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float2 *)ox,
-                                                                 (const float2 *)oy, (const float2 *)oz, nm,
-                                                                 p->n_rays, lm);
-            else
-                fwd_cone_kernel<4, true><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float4 *)ox,
-                                                                 (const float4 *)oy, (const float4 *)oz, nm,
-                                                                 p->n_rays, lm);
-        } else {
-            if (P == 1)
-                fwd_cone_kernel<1, false><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, ox, oy, oz, nm, p->n_rays,
-                                                                  lm);
-            else if (P == 2)
-                fwd_cone_kernel<2, false><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float2 *)ox,
-                                                                  (const float2 *)oy, (const float2 *)oz, nm,
-                                                                  p->n_rays, lm);
-            else
-                fwd_cone_kernel<4, false><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float4 *)ox,
-                                                                  (const float4 *)oy, (const float4 *)oz, nm,
-                                                                  p->n_rays, lm);
+        if (p->cols) {
+            PSPS_TRY(project_cone_cols(p, xm, lm, nm, s));
+            continue;
         }
+        const int P = nm == 1 ? 1 : (nm == 2 ? 2 : 4);
+        PSPS_TRY(cone_pack(p, xm, nm, P, true, s));
+        const float *ox = p->xcol.p, *oy = p->xrow.p, *oz = p->xcol3.p;
+        const unsigned gr = (unsigned)cdiv(p->n_rays, kThreads);
+        if (P == 1)
+            fwd_cone_kernel<1><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, ox, oy, oz, nm, p->n_rays, lm);
+        else if (P == 2)
+            fwd_cone_kernel<2><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float2 *)ox, (const float2 *)oy,
+                                                       (const float2 *)oz, nm, p->n_rays, lm);
+        else
+            fwd_cone_kernel<4><<<gr, kThreads, 0, s>>>(g, p->ray.p, p->ray3b.p, (const float4 *)ox, (const float4 *)oy,
+                                                       (const float4 *)oz, nm, p->n_rays, lm);
         PSPS_LAUNCH_CHECK();
     }
     return MBIR_OK;
@@ -1198,9 +1091,16 @@ mbir_status backproject_cone(mbir_plan *p, const float *sino, float *x, int n_ma
         PSPS_LAUNCH_CHECK();
         return MBIR_OK;
     }
-    // mode 0 (default): fixed-point tile scatter (the direct gather where the
-    // plan has no bound on the rays reaching a voxel); 1: direct gather; 3:
-    // split-table gather (1 and 3 bitwise equal)
+    // mode 0 (default): the column transpose; where it does not apply the
+    // fixed-point tile scatter (the direct gather where the plan has no bound
+    // on the rays reaching a voxel); 1: direct gather; 3: split-table gather
+    // (1 and 3 bitwise equal)
+    if (p->back_mode == 0 && p->col_rows > 0) {
+        for (int m0 = 0; m0 < n_mat; m0 += 4)
+            PSPS_TRY(backproject_cone_cols(p, sino + (int64_t)m0 * p->n_rays, x + (int64_t)m0 * p->n_pix,
+                                           n_mat - m0 < 4 ? n_mat - m0 : 4, accumulate, s));
+        return MBIR_OK;
+    }
     const int mode = p->back_mode == 0 && (p->cell_rays <= 0 || p->g.n_views > (1 << 20)) ? 1 : p->back_mode;
     const dim3 grd((unsigned)cdiv(p->g.nx, kGX), (unsigned)cdiv(p->g.ny, kGY), (unsigned)cdiv(p->g.nz, kGZ));
     const int tz = p->cone_tile == 8 ? 8 : 16;   // tile depth of the tile transpose

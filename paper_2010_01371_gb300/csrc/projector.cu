@@ -1251,8 +1251,7 @@ extern "C" mbir_status mbir_plan_create(const mbir_geometry *g, int n_mat_max, m
     p->n_pix = (int64_t)p->g.nx * p->g.ny * p->g.nz;
     mbir_status st;
     const int64_t copy = cone ? std::max<int64_t>(p->n_pix * 4, cone_pack_floats(p->g)) : p->n_pix * 4;
-    if ((st = p->xcol.alloc(copy)) != MBIR_OK || (st = p->xrow.alloc(copy)) != MBIR_OK ||
-        (cone && (st = p->xcol3.alloc(copy)) != MBIR_OK)) {
+    if ((st = p->xcol.alloc(copy)) != MBIR_OK || (st = p->xrow.alloc(copy)) != MBIR_OK) {
         delete p;
         return st;
     }
@@ -1384,14 +1383,15 @@ mbir_status autotune_impl(mbir_plan *p, int n_channels, cudaStream_t s) {
     PSPS_CUDA(cudaMemsetAsync(img.p, 0, sizeof(float) * img.n, s));
     float ms = 0.f, best_ms = 3.0e38f;
     if (p->g.kind == MBIR_CONE3D) {
-        // the transpose's algorithm: fixed-point tile scatter (0, where the
+        // the transpose's algorithm: detector columns or fixed-point tile
+        // scatter (0; the latter with tiles 16 or 8 voxels deep, where the
         // plan bounds the rays reaching a voxel), direct gather (1) or
-        // split-table gather (3)
-        // (the tile scatter with tiles 16 or 8 voxels deep)
+        // split-table gather (3); the forward has one algorithm
         int best = p->back_mode, best_tile = p->cone_tile;
         for (int cand : {0, 100, 1, 3}) {
             const int mode = cand == 100 ? 0 : cand;
-            if (mode == 0 && p->cell_rays <= 0) continue;
+            if (mode == 0 && p->cell_rays <= 0 && p->col_rows <= 0) continue;
+            if (cand == 100 && p->col_rows > 0) continue;   // the column transpose has no tile depth
             p->back_mode = mode;
             p->cone_tile = cand == 100 ? 8 : 16;
             PSPS_TRY(time_calls([&] { return backproject(p, sino.p, img.p, n_channels, 0, s); }, s, ev.e0, ev.e1, 1,
@@ -1400,15 +1400,6 @@ mbir_status autotune_impl(mbir_plan *p, int n_channels, cudaStream_t s) {
         }
         p->back_mode = best;
         p->cone_tile = best_tile;
-        // the forward's march: each lane from its own range (1) or warp-aligned (2)
-        best_ms = 3.0e38f;
-        best = p->fwd_mode;
-        for (int mode : {1, 2}) {
-            p->fwd_mode = mode;
-            PSPS_TRY(time_calls([&] { return project(p, img.p, sino.p, n_fwd, s); }, s, ev.e0, ev.e1, 1, ms));
-            if (ms < best_ms) best_ms = ms, best = mode;
-        }
-        p->fwd_mode = best;
         return MBIR_OK;
     }
     // 2-D transpose: views per CTA of the tile kernel
