@@ -154,12 +154,21 @@ __device__ inline void block_sum_partials_k(const dfloat *p, int n, double (&out
     dfloat a[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) a[k] = dfloat{0.f, 0.f};
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    // several loads of every stream in flight (their latency is all there is)
+    constexpr int U = K <= 4 ? 4 : 1;
+    for (int i = threadIdx.x; i < n; i += U * blockDim.x) {
+        float2 v[U][K];
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const float2 v = __ldcg(reinterpret_cast<const float2 *>(p + (size_t)k * n + i));
-            df_merge(a[k], dfloat{v.x, v.y});
-        }
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                v[u][k] = i + u * (int)blockDim.x < n
+                              ? __ldcg(reinterpret_cast<const float2 *>(p + (size_t)k * n + i + u * blockDim.x))
+                              : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < K; ++k) df_merge(a[k], dfloat{v[u][k].x, v[u][k].y});
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {

@@ -9,46 +9,12 @@
 #include <type_traits>
 
 #include "cone_cols.cuh"
+#include "f32x2.cuh"
 
 namespace psps {
 namespace {
 
 constexpr int kThreads = 256;
-
-// Pairs of FP32 values for the packed operations of sm_100 and later (two IEEE
-// operations per issue slot; the FMA rate itself is the scalar one, measured
-// 3.9 warp-wide FMAs per clock and SM either way, so the gain is in kernels
-// bound by instruction issue).
-using f32x2 = unsigned long long;
-
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
-__device__ __forceinline__ f32x2 pair2(float lo, float hi) {
-    f32x2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-
-__device__ __forceinline__ void unpair2(f32x2 v, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-
 
 // ------------------------------------------------------------------ packing
 

@@ -136,8 +136,7 @@ size_t spec_smem(SpecDev sp) { return sizeof(float) * (size_t)(sp.ne * sp.nm + s
 
 mbir_status launch_model_grad(SpecDev sp, int64_t n_rays, const float *l, const float *y, const float *gamma,
                               float *g, float *kappa, dfloat *partials, int nblocks, cudaStream_t s) {
-    const size_t smem = spec_smem(sp);
-    auto run = [&](auto fn) { fn(sp, n_rays, l, y, gamma, g, kappa, partials, nblocks, smem, s); };
+    auto run = [&](auto fn) { fn(sp, n_rays, l, y, gamma, g, kappa, partials, nblocks, s); };
     const bool rows = row_coupled(sp);
     switch (sp.nm) {
         case 1: rows ? run(model_rows_nm<1>) : run(model_grad_nm<1>); break;
@@ -152,8 +151,7 @@ mbir_status launch_model_grad(SpecDev sp, int64_t n_rays, const float *l, const 
 
 mbir_status launch_ls_fused(SpecDev sp, int64_t n_rays, const float *l, const float *q, const float *y, DevLS *ls,
                             LsCfg cfg, int mode, int last, dfloat *partials, int nblocks, cudaStream_t s) {
-    const size_t smem = spec_smem(sp);
-    auto run = [&](auto fn) { fn(sp, n_rays, l, q, y, ls, cfg, mode, last, partials, nblocks, smem, s); };
+    auto run = [&](auto fn) { fn(sp, n_rays, l, q, y, ls, cfg, mode, last, partials, nblocks, s); };
     const bool rows = row_coupled(sp);
     switch (sp.nm) {
         case 1: rows ? run(ls_rows_nm<1>) : run(ls_fused_nm<1>); break;

@@ -20,15 +20,39 @@ struct NoiseDev {
     int row = 1;
 };
 
+// Energy ranges between which the set of channels that see an energy (S > 0)
+// changes: photon-counting channels each see their own range, the channels of
+// a dual-kVp scan overlap only up to the lower voltage.  A channel's terms
+// outside its set are exact zeros, so leaving them out changes no sum.  n = 0:
+// one range, every channel.
+constexpr int kMaxSeg = 12;
+struct SpecSegs {
+    int n = 0;
+    int v[kMaxSeg] = {};   // first | end << 9 | channel mask << 18
+};
+
 struct SpecDev {
     int nm, ne, nc;
     const float *qs;  // Q[ne][nm], S[nc][ne], sigma[nc] (sigma_c = sum_E S[c][E])
     BlurDev blur;     // r = 0: no blur (b[0] = 1, the identity)
     NoiseDev noise;
+    SpecSegs segs;
 };
 
 inline SpecDev spec_dev(const mbmd_spectrum *s) {
-    SpecDev d{s->n_mat, s->n_energy, s->n_chan, s->qs.p, {}, {}};
+    SpecDev d{s->n_mat, s->n_energy, s->n_chan, s->qs.p, {}, {}, {}};
+    for (int e = 0; e < s->n_energy; ++e) {
+        int mask = 0;
+        for (int c = 0; c < s->n_chan; ++c) mask |= (float)s->hS[c * s->n_energy + e] != 0.f ? 1 << c : 0;
+        if (d.segs.n && d.segs.v[d.segs.n - 1] >> 18 == mask) {
+            d.segs.v[d.segs.n - 1] += 1 << 9;
+        } else if (d.segs.n == kMaxSeg) {
+            d.segs.n = 0;   // too many ranges: one, every channel
+            break;
+        } else {
+            d.segs.v[d.segs.n++] = e | (e + 1) << 9 | mask << 18;
+        }
+    }
     d.blur.r = s->blur_r;
     d.blur.row = s->blur_row;
     for (int k = 0; k < 7; ++k) d.blur.b[k] = s->blur_b[k];
@@ -42,13 +66,27 @@ inline SpecDev spec_dev(const mbmd_spectrum *s) {
 // and line-search kernels then work on row segments with halo rays.
 inline bool row_coupled(const SpecDev &sp) { return sp.blur.r > 0 || sp.noise.a > 0.f; }
 
-constexpr int kModelThreads = 256;
-constexpr int kModelMaxBlocks = 2048;  // grid-stride; partial sums per block
+constexpr int kModelThreads = 128;
+constexpr int kModelMaxBlocks = 2048;  // partial sums per block at most
 
-// About two rays per thread, at most kModelMaxBlocks blocks.
+// Two rays per thread at a time, a grid-stride loop over steps of 256 rays by
+// b blocks per SM: of b = 8 .. 5 (enough warps to keep the FP32 pipe busy) the
+// one that fills the last step best, since a nearly empty last step costs its
+// whole latency (720 x 888 rays, 2 materials, 121 energies, 2 channels: 152 us
+// for the line search with b = 8, whose third step holds 5 % of the blocks,
+// 147 with b = 6; 3 materials, 4 channels 257 and 236).
 inline int model_blocks(int64_t n) {
-    int64_t b = cdiv(n, 2 * kModelThreads);
-    return (int)(b < kModelMaxBlocks ? (b < 1 ? 1 : b) : kModelMaxBlocks);
+    const int64_t steps = cdiv(n, 2 * kModelThreads);
+    static_assert(152 * 8 <= kModelMaxBlocks, "partials");
+    if (steps <= 152 * 8) return (int)(steps < 1 ? 1 : steps);
+    int best = 8;
+    double fill = 0.0;
+    for (int b = 8; b >= 5; --b) {
+        const double s = (double)steps / (152.0 * b), f = s - (double)(int64_t)s;
+        const double last = (f == 0.0 ? 1.0 : f);
+        if (s < 32.0 && last > fill + 0.01) best = b, fill = last;
+    }
+    return 152 * best;
 }
 
 // data term partials (1 per block); g, kappa optional ([nm][n_rays]).
