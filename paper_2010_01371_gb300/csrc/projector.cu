@@ -31,6 +31,7 @@
 #include <cstring>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 
 namespace psps {
 namespace {
@@ -904,76 +905,129 @@ __global__ void __launch_bounds__(kThreads, 8)
 }
 
 // ---------------------------------------------------------------- strip forward
-// One CTA owns kSV consecutive views x kSB consecutive bins (one ray per
-// thread, lanes on neighbouring bins) and marches its rays through the image
-// in strips of S driving indices (columns for x-driven rays, rows for
-// y-driven ones).  For every strip the CTA finds the window of interpolated
-// indices its rays touch there (block min/max of the sample splits at the
-// strip ends; the split is monotone along a ray), stages that window of the
-// strip in shared memory (zero outside the image, so samples need no bounds
-// tests) and every lane then steps the same driving index: neighbouring lanes
-// read neighbouring shared-memory words.  Windows taller than kSH rows are
-// staged in part and the samples outside read global memory.  Sums: a plain
-// FP32 sum per strip (at most S samples), strips Kahan-compensated.  Weights
-// and the sample split are the per-ray table's, as in every other projector
-// and transpose, so the result is the same operator.
-// Views x bins per CTA: sb bins (a runtime choice among 32, 64, 128, 256,
-// tuned per plan) and kThreads / sb views, one ray per thread.
-constexpr int kSH = 256;           // staged window rows
+// One CTA owns kThreads / sb consecutive views x sb consecutive bins (one ray
+// per thread, lanes on neighbouring bins) and marches its rays through the
+// image in strips of S driving indices (columns for x-driven rays, rows for
+// y-driven ones).  Once per family and group of strips every ray's samples at
+// the ends of its part of a strip give, by warp and block minima, the window
+// of interpolated indices that the CTA touches there (the split is monotone
+// along a ray).  The window is staged in shared memory with 16-byte
+// asynchronous copies (zero outside the image, so samples need no bounds
+// tests), and every lane steps the same driving index: neighbouring lanes
+// read neighbouring shared-memory words, one wavefront per tap, where an
+// 8- or 16-byte gather through L1 costs four or eight for the cache lines its
+// lanes straddle.  A warp whose rays all cross the whole strip takes two
+// samples at a time as packed pairs at immediate offsets.  Windows taller
+// than kSH rows read the image in global memory.
+// Sums: a plain FP32 sum of at most kSub samples, those Kahan-compensated.
+// Weights and the sample split are the per-ray table's, as in every other
+// projector and transpose, so the result is the same operator.
+// Bound by issue (67-78 %) and shared-memory wavefronts (two or three per
+// sample and material).  512^2 from 720 x 888 rays, three images: 474 -> 389 us
+// against 16-byte gathers per ray, one image 171 -> 162; 448^2 from 720 x 780,
+// three images 387 -> 313.
+constexpr int kSH = 160;           // staged window rows
+constexpr int kStripGroup = 16;    // strips whose windows are found together
+constexpr int kSub = 16;           // samples per compensated add
 
 template <int NM>
 struct StripShape {
-    static constexpr int S = NM == 1 ? 32 : (NM == 2 ? 16 : 8);   // strip width (driving indices)
+    static constexpr int S = NM <= 2 ? 32 : 16;   // strip width (driving indices)
     static constexpr size_t smem = sizeof(float) * NM * S * kSH;
 };
 
-// Planar transposed copies xt[m][ix][iy] of x[m][iy][ix] (the x-driven
-// strips read columns contiguously), 32 x 32 tiles through shared memory.
-__global__ void transpose_planes_kernel(const float *__restrict__ x, int nm, int nx, int ny, float *__restrict__ xt) {
+// Row pitch of the copies that the strips are staged from: whole 16-byte
+// chunks, zero past the row's end.
+__host__ __device__ inline int strip_pitch(int n) { return (n + 3) & ~3; }
+
+// Planar transposed copies xt[m][ix][iy] of x[m][iy][ix] (the x-driven strips
+// read columns contiguously), 32 x 32 tiles through shared memory, and, when
+// xr is given, row copies xr[m][iy][ix], both with strip_pitch rows.
+__global__ void strip_pack_kernel(const float *__restrict__ x, int nx, int ny, float *__restrict__ xt,
+                                  float *__restrict__ xr) {
     __shared__ float tile[32][33];
     const int64_t npix = (int64_t)nx * ny;
     const int bx = blockIdx.x * 32, by = blockIdx.y * 32, m = blockIdx.z;
-    if (m >= nm) return;
+    const int px = strip_pitch(nx), py = strip_pitch(ny);
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int iy = by + r, ix = bx + threadIdx.x;
-        if (iy < ny && ix < nx) tile[r][threadIdx.x] = x[m * npix + (int64_t)iy * nx + ix];
+        const float v = iy < ny && ix < nx ? x[m * npix + (int64_t)iy * nx + ix] : 0.f;
+        tile[r][threadIdx.x] = v;
+        if (xr && iy < ny && ix < px) xr[((int64_t)m * ny + iy) * px + ix] = v;
     }
     __syncthreads();
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         const int ix = bx + r, iy = by + threadIdx.x;
-        if (iy < ny && ix < nx) xt[m * npix + (int64_t)ix * ny + iy] = tile[threadIdx.x][r];
+        if (iy < py && ix < nx) xt[((int64_t)m * nx + ix) * py + iy] = tile[threadIdx.x][r];
     }
 }
 
-__device__ __forceinline__ int block_min_int(int v, int *red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = min(r, red[w]);
-    return r;
+__device__ __forceinline__ void cp_async16(unsigned dst, const float *src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 
-__device__ __forceinline__ int block_max_int(int v, int *red) {
+template <int OFF>
+__device__ __forceinline__ float lds_off(unsigned a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(OFF));
+    return v;
+}
+
+template <int NM, int S, int c, int m>
+__device__ __forceinline__ void strip_taps(unsigned a0, unsigned a1, f32x2 f, f32x2 (&sum)[NM]) {
+    if constexpr (m < NM) {
+        constexpr int o0 = 4 * (m * S + c) * kSH, o1 = o0 + 4 * kSH;
+        const f32x2 a = pair2(lds_off<o0>(a0), lds_off<o1>(a1)), b = pair2(lds_off<o0 + 4>(a0), lds_off<o1 + 4>(a1));
+        sum[m] = add2(sum[m], fma2(f, sub2(b, a), a));
+        strip_taps<NM, S, c, m + 1>(a0, a1, f, sum);
+    }
+}
+
+// Samples c .. end - 1 (both even) of a strip that the whole warp crosses, two at a
+// time; base: shared-memory address of row 0's word of driving index 0 less
+// the split's integer offset.
+template <int NM, int S, int c, int end>
+__device__ __forceinline__ void strip_pairs(unsigned base, f32x2 fi, f32x2 df, f32x2 f0h, f32x2 (&sum)[NM]) {
+    if constexpr (c < end) {
+        const f32x2 magic = pair2(kSplitMagic, kSplitMagic);
+        const f32x2 h = fma2(fi, df, f0h), rn = add2(h, magic);
+        const f32x2 f = add2(sub2(h, sub2(rn, magic)), pair2(0.5f, 0.5f));
+        float r0, r1;
+        unpair2(rn, r0, r1);
+        const unsigned a0 = base + 4u * __float_as_uint(r0), a1 = base + 4u * __float_as_uint(r1);
+        strip_taps<NM, S, c, 0>(a0, a1, f, sum);
+        strip_pairs<NM, S, c + 2, end>(base, add2(fi, pair2(2.f, 2.f)), df, f0h, sum);
+    }
+}
+
+// The strip's S samples, kSub at a time.
+template <int NM, int S, int c, class Add>
+__device__ __forceinline__ void strip_sum(unsigned base, int i0, f32x2 df, f32x2 f0h, Add &&add) {
+    if constexpr (c < S) {
+        f32x2 sum[NM];
+        float v[NM];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int r = red[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = max(r, red[w]);
-    return r;
+        for (int m = 0; m < NM; ++m) sum[m] = 0ull;
+        strip_pairs<NM, S, c, c + kSub>(base, pair2((float)(i0 + c), (float)(i0 + c + 1)), df, f0h, sum);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            float a, b;
+            unpair2(sum[m], a, b);
+            v[m] = a + b;
+        }
+        add(v);
+        strip_sum<NM, S, c + kSub>(base, i0, df, f0h, add);
+    }
 }
 
 template <int NM>
-__global__ void __launch_bounds__(kThreads) fwd_strip_2d_kernel(const float4 *__restrict__ tab, mbir_geometry g,
-                                                                const float *__restrict__ x,
-                                                                const float *__restrict__ xt, int64_t n_rays, int sb,
-                                                                float *__restrict__ l) {
+__global__ void __launch_bounds__(kThreads, NM <= 2 ? 5 : 4)
+    fwd_strip_2d_kernel(const float4 *__restrict__ tab, mbir_geometry g, const float *__restrict__ xr,
+                        const float *__restrict__ xt, int64_t n_rays, int sb, float *__restrict__ l) {
     constexpr int S = StripShape<NM>::S;
-    extern __shared__ float sm[];   // [NM][S][kSH]
-    __shared__ int red[4][kThreads / 32];
-    const int tid = threadIdx.x;
+    extern __shared__ float4 strip_smem[];   // [NM][S][kSH] floats
+    __shared__ int wlo[kStripGroup], whi[kStripGroup], frange[2];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int view = blockIdx.y * (kThreads / sb) + tid / sb, bin = blockIdx.x * sb + tid % sb;
     const bool valid = view < g.n_views && bin < g.n_u;
     const int64_t ray = (int64_t)view * g.n_u + bin;
@@ -984,80 +1038,125 @@ __global__ void __launch_bounds__(kThreads) fwd_strip_2d_kernel(const float4 *__
         decode(r, axis, lo, hi);
     }
     const float f0h = r.x - 0.5f;
-    const int64_t npix = (int64_t)g.nx * g.ny;
+    const unsigned smem0 = (unsigned)__cvta_generic_to_shared(strip_smem);
     float acc[NM], comp[NM];
 #pragma unroll
     for (int m = 0; m < NM; ++m) acc[m] = comp[m] = 0.f;
+    auto add = [&](const float (&v)[NM]) {
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const float yk = __fsub_rn(v[m], comp[m]);
+            const float t = __fadd_rn(acc[m], yk);
+            comp[m] = __fsub_rn(__fsub_rn(t, acc[m]), yk);
+            acc[m] = t;
+        }
+    };
 #pragma unroll 1
     for (int fam = 0; fam < 2; ++fam) {
         const bool mine = valid && lo <= hi && axis == fam;
-        // driving-index range of this family's rays in the CTA (uniform)
-        const int f_lo = block_min_int(mine ? lo : INT_MAX, red[0]);
-        const int f_hi = block_max_int(mine ? hi : -1, red[1]);
+        // driving-index range of this family's rays in the CTA
+        if (tid == 0) frange[0] = INT_MAX, frange[1] = -1;
+        __syncthreads();
+        {
+            const int a = __reduce_min_sync(0xffffffffu, mine ? lo : INT_MAX);
+            const int b = __reduce_max_sync(0xffffffffu, mine ? hi : -1);
+            if (lane == 0 && b >= 0) atomicMin(&frange[0], a), atomicMax(&frange[1], b);
+        }
+        __syncthreads();
+        const int f_lo = frange[0], f_hi = frange[1];
         if (f_lo > f_hi) continue;
-        const int n_drive = fam == 0 ? g.nx : g.ny, n_other = fam == 0 ? g.ny : g.nx;
-        const float *src = fam == 0 ? xt : x;   // planar [m][driving][interpolated]
+        const int n_drive = fam == 0 ? g.nx : g.ny, n_other = fam == 0 ? g.ny : g.nx, pitch = strip_pitch(n_other);
+        const float *src = fam == 0 ? xt : xr;   // planar [m][driving][interpolated]
+        const int64_t plane = (int64_t)n_drive * pitch;
 #pragma unroll 1
-        for (int i0 = f_lo; i0 <= f_hi; i0 += S) {
-            const int ia = max(lo, i0), ib = min(hi, i0 + S - 1);
-            const bool has = mine && ia <= ib;
-            int ka = INT_MAX, kb = INT_MIN;
-            if (has) {
-                float fa, fb;
-                const int k1 = joseph_split(fmaf((float)ia, r.y, f0h), fa);
-                const int k2 = joseph_split(fmaf((float)ib, r.y, f0h), fb);
-                ka = min(k1, k2) - 1;       // one index of margin on each side
-                kb = max(k1, k2) + 2;       // upper neighbour k + 1, plus margin
-            }
-            __syncthreads();   // previous strip's readers of sm and red are done
-            const int w0 = block_min_int(ka, red[2]);
-            const int w1 = block_max_int(kb, red[3]);
-            if (w1 < w0) continue;                  // no ray of the CTA samples this strip
-            const int hs = min(w1 - w0 + 1, kSH);   // staged rows [w0, w0 + hs)
-            // one warp per (material, strip index), lanes down the window
-            for (int mc = tid >> 5; mc < NM * S; mc += kThreads / 32) {
-                const int m = mc / S, i = i0 + (mc - m * S);
-                const float *col = src + m * npix + (int64_t)i * n_other;
-                float *dst = sm + mc * kSH;
-                const bool in_i = i < n_drive;
-                for (int rr = tid & 31; rr < hs; rr += 32) {
-                    const int row = w0 + rr;
-                    dst[rr] = (in_i && row >= 0 && row < n_other) ? __ldg(col + row) : 0.f;
+        for (int g0 = f_lo; g0 <= f_hi; g0 += S * kStripGroup) {
+            if (tid < kStripGroup) wlo[tid] = INT_MAX, whi[tid] = INT_MIN;
+            __syncthreads();
+            // Lane q: strip q, over this warp's rays of the family.  Their
+            // positions on a driving index are monotone in the bin, so the
+            // first and the last ray bound them, at the ends of the strip's
+            // part that any of them covers (one row of margin for rounding).
+            const unsigned rays = __ballot_sync(0xffffffffu, mine);
+            if (rays) {
+                const int first = __ffs(rays) - 1, last = 31 - __clz(rays);
+                const float xa = __shfl_sync(0xffffffffu, f0h, first), sa = __shfl_sync(0xffffffffu, r.y, first);
+                const float xb = __shfl_sync(0xffffffffu, f0h, last), sb2 = __shfl_sync(0xffffffffu, r.y, last);
+                const int w_lo = __reduce_min_sync(0xffffffffu, mine ? lo : INT_MAX);
+                const int w_hi = __reduce_max_sync(0xffffffffu, mine ? hi : -1);
+                const int i0 = g0 + lane * S, ia = max(w_lo, i0), ib = min(w_hi, i0 + S - 1);
+                if (lane < kStripGroup && ia <= ib) {
+                    float f;
+                    const int k0 = joseph_split(fmaf((float)ia, sa, xa), f), k1 = joseph_split(fmaf((float)ib, sa, xa), f);
+                    const int k2 = joseph_split(fmaf((float)ia, sb2, xb), f), k3 = joseph_split(fmaf((float)ib, sb2, xb), f);
+                    atomicMin(&wlo[lane], min(min(k0, k1), min(k2, k3)) - 1);
+                    atomicMax(&whi[lane], max(max(k0, k1), max(k2, k3)) + 2);
                 }
             }
             __syncthreads();
-            if (has) {
-                float sum[NM];
-#pragma unroll
-                for (int m = 0; m < NM; ++m) sum[m] = 0.f;
-                for (int i = ia; i <= ib; ++i) {
-                    float f;
-                    const int k = joseph_split(fmaf((float)i, r.y, f0h), f);
-                    const int kl = k - w0, c = i - i0;
-                    if (kl >= 0 && kl + 1 < hs) {
-#pragma unroll
-                        for (int m = 0; m < NM; ++m) {
-                            const float a = sm[(m * S + c) * kSH + kl], b = sm[(m * S + c) * kSH + kl + 1];
-                            sum[m] += fmaf(f, b - a, a);
-                        }
-                    } else {
-                        // outside the staged part of a tall window
-#pragma unroll
-                        for (int m = 0; m < NM; ++m) {
-                            const float *col = src + m * npix + (int64_t)i * n_other;
-                            const float a = (k >= 0 && k < n_other) ? __ldg(col + k) : 0.f;
-                            const float b = (k + 1 >= 0 && k + 1 < n_other) ? __ldg(col + k + 1) : 0.f;
-                            sum[m] += fmaf(f, b - a, a);
+#pragma unroll 1
+            for (int q = 0; q < kStripGroup; ++q) {
+                const int w1 = whi[q];
+                if (w1 == INT_MIN) continue;                 // no ray of the CTA samples this strip
+                const int i0 = g0 + q * S, w0 = wlo[q] & ~3; // whole chunks
+                const int hs = w1 - w0 + 1;
+                const bool staged = hs <= kSH;
+                if (staged)                                  // a warp per (material, driving index)
+                    for (int mc = wid; mc < NM * S; mc += kThreads / 32) {
+                        const int m = mc / S, i = i0 + (mc - m * S);
+                        const float *row = src + m * plane + (int64_t)i * pitch;
+                        for (int c = 4 * lane; c < hs; c += 128) {
+                            const int k = w0 + c;
+                            const bool in = i < n_drive && k >= 0 && k < pitch;
+                            cp_async16(smem0 + 4u * (mc * kSH + c), in ? row + k : src, in);
                         }
                     }
-                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncthreads();
+                const int ia = max(lo, i0), ib = min(hi, i0 + S - 1);
+                const bool has = mine && ia <= ib;
+                if (staged) {
+                    // base + 4 * (bits of the rounded coordinate) is the address of row k's word
+                    const unsigned base = smem0 - 4u * (unsigned)(__float_as_int(kSplitMagic) + w0);
+                    if (__all_sync(0xffffffffu, has && ia == i0 && ib == i0 + S - 1)) {
+                        const f32x2 df = pair2(r.y, r.y), f0 = pair2(f0h, f0h);
+                        strip_sum<NM, S, 0>(base, i0, df, f0, add);
+                    } else if (has) {
+                        float v[NM];
 #pragma unroll
-                for (int m = 0; m < NM; ++m) {
-                    const float yk = __fsub_rn(sum[m], comp[m]);
-                    const float t = __fadd_rn(acc[m], yk);
-                    comp[m] = __fsub_rn(__fsub_rn(t, acc[m]), yk);
-                    acc[m] = t;
+                        for (int m = 0; m < NM; ++m) v[m] = 0.f;
+                        for (int i = ia; i <= ib; ++i) {
+                            const float h = fmaf((float)i, r.y, f0h), rn = h + kSplitMagic;
+                            const float f = (h - (rn - kSplitMagic)) + 0.5f;
+                            const unsigned a0 = base + 4u * __float_as_uint(rn) + 4u * kSH * (unsigned)(i - i0);
+#pragma unroll
+                            for (int m = 0; m < NM; ++m) {
+                                const float *p = reinterpret_cast<const float *>(
+                                    reinterpret_cast<const char *>(strip_smem) + (a0 - smem0) + 4 * m * S * kSH);
+                                v[m] += fmaf(f, p[1] - p[0], p[0]);
+                            }
+                            if ((i - ia) % kSub == kSub - 1) {
+                                add(v);
+#pragma unroll
+                                for (int m = 0; m < NM; ++m) v[m] = 0.f;
+                            }
+                        }
+                        add(v);
+                    }
+                } else if (has) {
+                    for (int i = ia; i <= ib; ++i) {
+                        float f, v[NM];
+                        const int k = joseph_split(fmaf((float)i, r.y, f0h), f);
+#pragma unroll
+                        for (int m = 0; m < NM; ++m) {
+                            const float *col = src + m * plane + (int64_t)i * pitch;
+                            const float a = (k >= 0 && k < n_other) ? __ldg(col + k) : 0.f;
+                            const float b = (k + 1 >= 0 && k + 1 < n_other) ? __ldg(col + k + 1) : 0.f;
+                            v[m] = fmaf(f, b - a, a);
+                        }
+                        add(v);
+                    }
                 }
+                __syncthreads();   // the strip's readers are done
             }
         }
     }
@@ -1069,13 +1168,18 @@ __global__ void __launch_bounds__(kThreads) fwd_strip_2d_kernel(const float4 *__
 template <int NM>
 mbir_status project_strip_nm(mbir_plan *p, const float *x, float *l, cudaStream_t s) {
     const int nx = p->g.nx, ny = p->g.ny;
+    // the image itself serves as its row copy when its rows are whole chunks
+    const bool direct = nx % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     const dim3 tb(32, 8), tg((unsigned)cdiv(nx, 32), (unsigned)cdiv(ny, 32), (unsigned)NM);
-    transpose_planes_kernel<<<tg, tb, 0, s>>>(x, NM, nx, ny, p->xcol.p);
+    strip_pack_kernel<<<tg, tb, 0, s>>>(x, nx, ny, p->xcol.p, direct ? nullptr : p->xrow.p);
     PSPS_LAUNCH_CHECK();
     const int sb = p->strip_bins, sv = kThreads / sb;
     const dim3 grd((unsigned)cdiv(p->g.n_u, sb), (unsigned)cdiv(p->g.n_views, sv));
-    fwd_strip_2d_kernel<NM><<<grd, kThreads, StripShape<NM>::smem, s>>>(p->ray.p, p->g, x, p->xcol.p, p->n_rays, sb,
-                                                                        l);
+    if (StripShape<NM>::smem > 40 * 1024)
+        PSPS_CUDA(cudaFuncSetAttribute(fwd_strip_2d_kernel<NM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)StripShape<NM>::smem));
+    fwd_strip_2d_kernel<NM><<<grd, kThreads, StripShape<NM>::smem, s>>>(p->ray.p, p->g, direct ? x : p->xrow.p,
+                                                                        p->xcol.p, p->n_rays, sb, l);
     PSPS_LAUNCH_CHECK();
     return MBIR_OK;
 }
@@ -1111,6 +1215,12 @@ mbir_status project_2d_nm(mbir_plan *p, const float *x, float *l, cudaStream_t s
 
 }  // namespace
 
+// Angle between the outer rays of a warp of the strip forward (their
+// positions are then monotone in the bin); wider ones go ray by ray.
+static double strip_bins_span(const mbir_plan *p) {
+    return p->g.kind == MBIR_PAR2D ? 0.0 : 32.0 * p->g.du / p->g.sdd;
+}
+
 mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStream_t s) {
     if (p->g.kind == MBIR_CONE3D) return project_cone(p, x, l, n_mat, s);
     if (p->fwd_mode == 0) {
@@ -1137,7 +1247,7 @@ mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStrea
         const int nm = n_mat - m0 < 4 ? n_mat - m0 : 4;
         const float *xm = x + (int64_t)m0 * p->n_pix;
         float *lm = l + (int64_t)m0 * p->n_rays;
-        if (p->fwd_mode == 2) {
+        if (p->fwd_mode == 2 && strip_bins_span(p) < 1.5) {
             switch (nm) {
                 case 1: PSPS_TRY(project_strip_nm<1>(p, xm, lm, s)); break;
                 case 2: PSPS_TRY(project_strip_nm<2>(p, xm, lm, s)); break;
@@ -1250,7 +1360,9 @@ extern "C" mbir_status mbir_plan_create(const mbir_geometry *g, int n_mat_max, m
     p->n_rays = (int64_t)p->g.n_views * p->g.n_u * p->g.n_v;
     p->n_pix = (int64_t)p->g.nx * p->g.ny * p->g.nz;
     mbir_status st;
-    const int64_t copy = cone ? std::max<int64_t>(p->n_pix * 4, cone_pack_floats(p->g)) : p->n_pix * 4;
+    const int64_t copy =
+        cone ? std::max<int64_t>(p->n_pix * 4, cone_pack_floats(p->g))
+             : 4 * std::max((int64_t)g->nx * strip_pitch(g->ny), (int64_t)g->ny * strip_pitch(g->nx));
     if ((st = p->xcol.alloc(copy)) != MBIR_OK || (st = p->xrow.alloc(copy)) != MBIR_OK) {
         delete p;
         return st;
@@ -1282,6 +1394,23 @@ extern "C" mbir_status mbir_plan_create(const mbir_geometry *g, int n_mat_max, m
             if (p->g.sid > R) delta = (p->g.sid - R) * (p->g.du / p->g.sdd) / pix;
         }
         p->cell_rays = delta > 1e-3 ? (int)std::floor(2.0 / delta) + 2 : 0;
+    }
+    {
+        // Forward: the strips (32 bins x 8 views per CTA) where there are
+        // enough CTAs to hide their staging (about eight per SM) and a CTA's
+        // window fits the staged rows, one thread per ray otherwise.  Measured
+        // (us, per ray / strips): 512^2 from 720 x 888 rays, one image 171 / 162,
+        // three 474 / 389; 320^2 from 720 x 556 86 / 86 and 235 / 188; 256^2 from
+        // 360 x 444 (630 CTAs) 41 / 58 and 93 / 99.  On a driving plane adjacent
+        // rays are at most sqrt2 du (1 + R / sid) sid / sdd / pixel apart (fan;
+        // du for parallel beam), a ray moves at most one row per driving index,
+        // and the CTA's views turn by their spacing each.
+        const mbir_geometry &q = p->g;
+        const double pix = std::min(q.dx, q.dy), R = std::hypot(0.5 * q.nx * q.dx, 0.5 * q.ny * q.dy);
+        const double d = std::sqrt(2.0) * (q.kind == MBIR_PAR2D ? q.du : q.du * (q.sid + R) / q.sdd) / pix;
+        const double turn = std::sqrt(2.0) * R / pix * std::fabs(q.angle_span) / q.n_views;
+        const int64_t ctas = cdiv(q.n_u, 32) * cdiv(q.n_views, kThreads / 32);
+        if (ctas >= 152 * 8 && 32 * d + (kThreads / 32 - 1) * turn + 32.0 + 8.0 <= kSH) p->fwd_mode = 2, p->strip_bins = 32;
     }
     {
         // default views per CTA of the tile transpose: about six CTAs per SM
