@@ -38,6 +38,24 @@ __device__ inline bool last_block_arrive(unsigned *ticket) {
     return last;
 }
 
+// phi(0) = data + 1/2 x.Rx, recorded in the objective history.
+__device__ inline void ls_begin(DevLS *ls, double data, double xRx, double *history) {
+    ls->R0 = 0.5 * xRx;
+    ls->phi0 = data + 0.5 * xRx;
+    if (!isfinite(ls->phi0)) ls->nonfinite = 1;
+    history[ls->it] = ls->phi0;
+}
+
+// Start of a search along p (penalty terms p.Rx, p.Rp).
+__device__ inline void ls_init(DevLS *ls, double pRx, double pRp) {
+    ls->pRx = pRx;
+    ls->pRp = pRp;
+    ls->alpha = ls->a_prev > 0 ? ls->a_prev : 1.0;
+    ls->best_a = 0.0;
+    ls->best_f = INFINITY;
+    ls->done = 0;
+}
+
 // One Newton evaluation (phi, phi', phi'' data sums; bad = rays outside the
 // domain) at ls->alpha; the last one decides acceptance.
 __device__ inline void ls_newton_control(DevLS *ls, double fd, double f1d, double f2d, double bad, int last,

@@ -29,7 +29,8 @@ __device__ __forceinline__ float gamma_at(const float *__restrict__ v, int64_t j
 // abs_mode: |R| v instead (positive taps, |beta|), no reductions.
 __global__ void __launch_bounds__(kThreads)
     penalty_kernel(PenaltyDev pd, int nx, int ny, int nz, const float *__restrict__ x, const float *__restrict__ p,
-                   float *__restrict__ rx_out, int accumulate, int abs_mode, dfloat *__restrict__ partials) {
+                   float *__restrict__ rx_out, int accumulate, int abs_mode, dfloat *__restrict__ partials,
+                   PenaltyCtl ctl) {
     const int64_t npix = (int64_t)nx * ny * nz;
     dfloat s0{0.f, 0.f}, s1{0.f, 0.f}, s2{0.f, 0.f};
     const float sign = abs_mode ? 1.f : -1.f;
@@ -69,13 +70,25 @@ __global__ void __launch_bounds__(kThreads)
         dfloat v[3] = {s0, s1, s2};
         block_sum_store<3>(v, partials);
     }
+    if (ctl.then == kPenaltyOnly || !last_block_arrive(&ctl.ls->ticket)) return;
+    const int nb = gridDim.x;
+    if (ctl.then == kPenaltyBegin) {
+        const double data = block_sum_partials(ctl.pobj, ctl.nobj), xRx = block_sum_partials(partials, nb);
+        if (threadIdx.x == 0) ls_begin(ctl.ls, data, xRx, ctl.history);
+    } else {
+        double pen[2];
+        block_sum_partials_k<2>(partials + nb, nb, pen);
+        if (threadIdx.x == 0) ls_init(ctl.ls, pen[0], pen[1]);
+    }
+    if (threadIdx.x == 0) ctl.ls->ticket = 0;
 }
 
 }  // namespace
 
 mbir_status launch_penalty(const PenaltyDev &pd, int nx, int ny, int nz, const float *x, const float *p, float *rx_out,
-                           int accumulate, int abs_mode, dfloat *partials, int nblocks, cudaStream_t s) {
-    penalty_kernel<<<nblocks, kThreads, 0, s>>>(pd, nx, ny, nz, x, p, rx_out, accumulate, abs_mode, partials);
+                           int accumulate, int abs_mode, dfloat *partials, int nblocks, const PenaltyCtl &ctl,
+                           cudaStream_t s) {
+    penalty_kernel<<<nblocks, kThreads, 0, s>>>(pd, nx, ny, nz, x, p, rx_out, accumulate, abs_mode, partials, ctl);
     PSPS_LAUNCH_CHECK();
     return MBIR_OK;
 }

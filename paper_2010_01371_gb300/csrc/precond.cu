@@ -489,7 +489,7 @@ struct HessOp {
         if (has_pen)
             for (int p = 0; p < nprobe; ++p)
                 PSPS_TRY(launch_penalty(pd, plan->g.nx, plan->g.ny, plan->g.nz, v + (int64_t)p * nm * n, nullptr,
-                                        out + (int64_t)p * nm * n, 1, 0, nullptr, penalty_blocks(n), s));
+                                        out + (int64_t)p * nm * n, 1, 0, nullptr, penalty_blocks(n), PenaltyCtl{}, s));
         return MBIR_OK;
     }
 };
@@ -692,6 +692,13 @@ mbir_status precond_apply(psps_precond *pc, int op, const float *in, float *out,
 
 mbir_status precond_apply2(psps_precond *pc, int op0, const float *in0, float *out0, int op1, const float *in1,
                            float *out1, cudaStream_t s) {
+    // M^T and |M|^T of one wavelet preconditioner over consecutive channels:
+    // one apply, |U| for the upper half (M0 enters both alike)
+    const int64_t tot = pc->n * pc->nm;
+    if (pc->kind == PSPS_PRECOND_HAAR && op0 == PSPS_APPLY_MT && op1 == PSPS_APPLY_ABS_MT && in1 == in0 + tot &&
+        out1 == out0 + tot)
+        return haar_apply(pc->nx, 2 * pc->nm, in0, pc->tmp.p, out0, pc->m0.p, pc->sides == 2 ? pc->m0.p : nullptr,
+                          pc->s.p, ((1u << pc->nm) - 1u) << pc->nm, s, pc->nz);
     PSPS_TRY(precond_apply(pc, op0, in0, out0, s));
     return precond_apply(pc, op1, in1, out1, s);
 }

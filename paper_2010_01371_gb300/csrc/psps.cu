@@ -30,30 +30,15 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// phi0 = data + 1/2 x.Rx; records the objective history.
-__global__ void ctrl_begin_kernel(DevLS *ls, const dfloat *pobj, int nobj, const dfloat *ppen, int npen,
-                                  double *history) {
+// phi0 and the objective history without a penalty (with one, the penalty
+// kernel's last block does it); then, for an iteration, the line search's
+// starting point (search) or the unit step.
+__global__ void ctrl_begin_kernel(DevLS *ls, const dfloat *pobj, int nobj, double *history, int iteration, int search) {
     const double d = block_sum_partials(pobj, nobj);
-    const double xRx = ppen ? block_sum_partials(ppen, npen) : 0.0;
     if (threadIdx.x == 0) {
-        ls->R0 = 0.5 * xRx;
-        ls->phi0 = d + 0.5 * xRx;
-        if (!isfinite(ls->phi0)) ls->nonfinite = 1;
-        history[ls->it] = ls->phi0;
-    }
-}
-
-// penalty terms along p: partials are (x.Rx, p.Rx, p.Rp) blocks
-__global__ void ctrl_ls_init_kernel(DevLS *ls, const dfloat *ppen, int npen) {
-    double pen[2] = {0.0, 0.0};
-    if (ppen) block_sum_partials_k<2>(ppen + npen, npen, pen);
-    if (threadIdx.x == 0) {
-        ls->pRx = pen[0];
-        ls->pRp = pen[1];
-        ls->alpha = ls->a_prev > 0 ? ls->a_prev : 1.0;
-        ls->best_a = 0.0;
-        ls->best_f = INFINITY;
-        ls->done = 0;
+        ls_begin(ls, d, 0.0, history);
+        if (iteration && search) ls_init(ls, 0.0, 0.0);
+        if (iteration && !search) ls->alpha = 1.0;
     }
 }
 
@@ -68,11 +53,18 @@ __global__ void direction_kernel(const float *__restrict__ gp, const float *__re
     }
 }
 
-// x += alpha p (clamped at 0 when nonneg), l += alpha q; records alpha
+// x += alpha p (clamped at 0 when nonneg), l += alpha q; records alpha (one
+// thread; the other blocks read none of what it writes).  The next line
+// search starts from it, or below the last halving after a failed search.
 __global__ void update_kernel(DevLS *ls, float *__restrict__ x, const float *__restrict__ p, int64_t nx_tot,
                               float *__restrict__ l, const float *__restrict__ q, int64_t nl_tot, int nonneg,
-                              double *alphas) {
+                              double *alphas, int n_halve) {
     const float a = (float)ls->alpha;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        alphas[ls->it] = ls->alpha;
+        ls->a_prev = ls->alpha > 0 ? ls->alpha : ls->best_a / (double)(2 << n_halve);
+        ls->it += 1;
+    }
     const int64_t tot = nx_tot > nl_tot ? nx_tot : nl_tot;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
         if (i < nx_tot) {
@@ -82,14 +74,6 @@ __global__ void update_kernel(DevLS *ls, float *__restrict__ x, const float *__r
         }
         if (l && i < nl_tot) l[i] = fmaf(a, q[i], l[i]);
     }
-}
-
-// Records alpha; the next line search starts from it, or below the last
-// halving after a failed search.
-__global__ void finish_iter_kernel(DevLS *ls, double *alphas, int n_halve) {
-    alphas[ls->it] = ls->alpha;
-    ls->a_prev = ls->alpha > 0 ? ls->alpha : ls->best_a / (double)(2 << n_halve);
-    ls->it += 1;
 }
 
 __global__ void reset_counter_kernel(DevLS *ls) {
@@ -116,7 +100,7 @@ struct psps_state {
     bool has_pen = false;
     PenaltyDev pd{};
     LsCfg cfg{3, 8, 1e12, 8.0, -20.0f};
-    DBuf<float> x, l, y, gamma, dR, gk, G, gp, dp, pp, p, q;
+    DBuf<float> x, l, y, gamma, dR, gk, G, gp, pp, p, q;   // gp: [grad'; d']
     SpecDev sd;  // the spectrum (and its blur) as it was at creation
     DBuf<dfloat> part_obj, part_pen, part_ls;
     DBuf<double> history, alphas;
@@ -192,10 +176,21 @@ mbir_status apply_M(psps_state *st, int op, const float *in, float *out, cudaStr
 }
 
 mbir_status penalty_call(psps_state *st, const float *x, const float *p, float *rx_out, int acc, int abs_mode,
-                         dfloat *part, cudaStream_t s) {
+                         dfloat *part, int then, cudaStream_t s) {
     const mbir_geometry &g = st->plan->g;
+    const PenaltyCtl ctl{then, st->ls.p, st->part_obj.p, st->nb_model, st->history.p};
     return launch_penalty(st->pd, g.nx, g.ny, g.kind == MBIR_CONE3D ? g.nz : 1, x, p, rx_out, acc, abs_mode, part,
-                          st->nb_pen, s);
+                          st->nb_pen, ctl, s);
+}
+
+// phi(0) into the history: the penalty pass adds x.Rx (and R x to grad, if
+// given) and its last block closes the sums; without a penalty one block does.
+mbir_status begin(psps_state *st, float *grad, int iteration, cudaStream_t s) {
+    if (st->has_pen) return penalty_call(st, st->x.p, nullptr, grad, 1, 0, st->part_pen.p, kPenaltyBegin, s);
+    ctrl_begin_kernel<<<1, kThreads, 0, s>>>(st->ls.p, st->part_obj.p, st->nb_model, st->history.p, iteration,
+                                             st->flags & PSPS_FLAG_LINESEARCH);
+    PSPS_LAUNCH_CHECK();
+    return MBIR_OK;
 }
 
 // One iteration (no host synchronisation).
@@ -221,15 +216,16 @@ mbir_status iterate(psps_state *st, bool reproject, cudaStream_t s) {
     PSPS_TRY(backproject_or_copy(st, st->gk.p, st->G.p, 2 * nm, s, fine ? nm : 0));
     mark(st, PSPS_PROF_BACKPROJECT, 1, s);
     mark(st, PSPS_PROF_PRECOND, 0, s);
-    if (st->has_pen) PSPS_TRY(penalty_call(st, st->x.p, nullptr, st->G.p, 1, 0, st->part_pen.p, s));
-    ctrl_begin_kernel<<<1, kThreads, 0, s>>>(st->ls.p, st->part_obj.p, st->nb_model,
-                                             st->has_pen ? st->part_pen.p : nullptr, st->nb_pen, st->history.p);
-    PSPS_LAUNCH_CHECK();
+    PSPS_TRY(begin(st, st->G.p, 1, s));
     // preconditioned gradient, curvature and direction
-    PSPS_TRY(apply_M(st, PSPS_APPLY_MT, st->G.p, st->gp.p, s));
-    PSPS_TRY(apply_M(st, PSPS_APPLY_ABS_MT, st->G.p + (int64_t)nm * n, st->dp.p, s));
-    direction_kernel<<<grid_for(nm * n), kThreads, 0, s>>>(st->gp.p, st->dp.p, st->has_pen ? st->dR.p : nullptr,
-                                                           st->pp.p, nm * n);
+    float *const gp = st->gp.p, *const dp = gp + (int64_t)nm * n, *const curv = st->G.p + (int64_t)nm * n;
+    if (st->pc) {
+        PSPS_TRY(precond_apply2(st->pc, PSPS_APPLY_MT, st->G.p, gp, PSPS_APPLY_ABS_MT, curv, dp, s));
+    } else {
+        PSPS_TRY(apply_M(st, PSPS_APPLY_MT, st->G.p, gp, s));
+        PSPS_TRY(apply_M(st, PSPS_APPLY_ABS_MT, curv, dp, s));
+    }
+    direction_kernel<<<grid_for(nm * n), kThreads, 0, s>>>(gp, dp, st->has_pen ? st->dR.p : nullptr, st->pp.p, nm * n);
     PSPS_LAUNCH_CHECK();
     PSPS_TRY(apply_M(st, PSPS_APPLY_M, st->pp.p, st->p.p, s));
     mark(st, PSPS_PROF_PRECOND, 1, s);
@@ -240,9 +236,8 @@ mbir_status iterate(psps_state *st, bool reproject, cudaStream_t s) {
     // step length
     mark(st, PSPS_PROF_LINESEARCH, 0, s);
     if (st->flags & PSPS_FLAG_LINESEARCH) {
-        if (st->has_pen) PSPS_TRY(penalty_call(st, st->x.p, st->p.p, nullptr, 0, 0, st->part_pen.p, s));
-        ctrl_ls_init_kernel<<<1, kThreads, 0, s>>>(st->ls.p, st->has_pen ? st->part_pen.p : nullptr, st->nb_pen);
-        PSPS_LAUNCH_CHECK();
+        // without a penalty the search was set up with phi(0)
+        if (st->has_pen) PSPS_TRY(penalty_call(st, st->x.p, st->p.p, nullptr, 0, 0, st->part_pen.p, kPenaltySearch, s));
         const int nb = st->nb_model;
         for (int k = 0; k < st->cfg.n_ls; ++k)
             PSPS_TRY(launch_ls_fused(sp, nr, st->l.p, st->q.p, st->y.p, st->ls.p, st->cfg, 0, k + 1 == st->cfg.n_ls,
@@ -250,7 +245,7 @@ mbir_status iterate(psps_state *st, bool reproject, cudaStream_t s) {
         if (st->cfg.n_halve > 0)
             PSPS_TRY(
                 launch_ls_fused(sp, nr, st->l.p, st->q.p, st->y.p, st->ls.p, st->cfg, 1, 1, st->part_ls.p, nb, s));
-    } else {
+    } else if (st->has_pen) {
         set_alpha_one_kernel<<<1, 1, 0, s>>>(st->ls.p);
         PSPS_LAUNCH_CHECK();
     }
@@ -258,9 +253,7 @@ mbir_status iterate(psps_state *st, bool reproject, cudaStream_t s) {
     mark(st, PSPS_PROF_UPDATE, 0, s);
     update_kernel<<<grid_for(nm * (n > nr ? n : nr)), kThreads, 0, s>>>(
         st->ls.p, st->x.p, st->p.p, nm * n, nonneg ? nullptr : st->l.p, st->q.p, nm * nr, nonneg ? 1 : 0,
-        st->alphas.p);
-    PSPS_LAUNCH_CHECK();
-    finish_iter_kernel<<<1, 1, 0, s>>>(st->ls.p, st->alphas.p, st->cfg.n_halve);
+        st->alphas.p, st->cfg.n_halve);
     PSPS_LAUNCH_CHECK();
     if (nonneg) PSPS_TRY(project_or_copy(st, st->x.p, st->l.p, s));
     mark(st, PSPS_PROF_UPDATE, 1, s);
@@ -271,11 +264,7 @@ mbir_status final_objective(psps_state *st, cudaStream_t s) {
     PSPS_TRY(project_or_copy(st, st->x.p, st->l.p, s));
     PSPS_TRY(launch_model_grad(st->sd, st->n_rays, st->l.p, st->y.p, nullptr, nullptr, nullptr,
                                st->part_obj.p, st->nb_model, s));
-    if (st->has_pen) PSPS_TRY(penalty_call(st, st->x.p, nullptr, nullptr, 0, 0, st->part_pen.p, s));
-    ctrl_begin_kernel<<<1, kThreads, 0, s>>>(st->ls.p, st->part_obj.p, st->nb_model,
-                                             st->has_pen ? st->part_pen.p : nullptr, st->nb_pen, st->history.p);
-    PSPS_LAUNCH_CHECK();
-    return MBIR_OK;
+    return begin(st, nullptr, 0, s);
 }
 
 // Kernel nodes of a captured graph (the launches one replay makes).
@@ -373,8 +362,7 @@ extern "C" mbir_status psps_state_create(mbir_plan *plan, const mbmd_spectrum *s
     A(st->dR, nm * n);
     A(st->gk, 2 * nm * nr);
     A(st->G, 2 * nm * n);
-    A(st->gp, nm * n);
-    A(st->dp, nm * n);
+    A(st->gp, 2 * nm * n);
     A(st->pp, nm * n);
     A(st->p, nm * n);
     A(st->q, nm * nr);
@@ -402,7 +390,7 @@ extern "C" mbir_status psps_state_create(mbir_plan *plan, const mbmd_spectrum *s
         PSPS_TRY(project_or_copy(st, absM1, st->gamma.p, s));
         PSPS_CUDA(cudaMemsetAsync(st->dR.p, 0, sizeof(float) * nm * n, s));
         if (st->has_pen) {
-            PSPS_TRY(penalty_call(st, absM1, nullptr, st->gp.p, 0, 1, nullptr, s));
+            PSPS_TRY(penalty_call(st, absM1, nullptr, st->gp.p, 0, 1, nullptr, kPenaltyOnly, s));
             PSPS_TRY(apply_M(st, PSPS_APPLY_ABS_MT, st->gp.p, st->dR.p, s));
         }
         PSPS_TRY(project_or_copy(st, st->x.p, st->l.p, s));
