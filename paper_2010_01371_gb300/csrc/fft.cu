@@ -29,6 +29,15 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// x / d for x, d < 2^16 with one multiply (an integer division takes about 20
+// instructions, and a pass made three per butterfly): floor(x m / 2^32) with
+// m = floor((2^32 - 1) / d) + 1 is exact there; d = 1 has no such m.
+struct FastDiv {
+    unsigned m;
+    __device__ __forceinline__ explicit FastDiv(int d) : m(d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u) {}
+    __device__ __forceinline__ int div(int x) const { return m ? (int)__umulhi((unsigned)x, m) : x; }
+};
+
 // Roots of unity of the small DFTs, stored after the N twiddles of a table:
 // offsets of the R = 3, 5, 7 roots e^{-2 pi i k/R}, k < R.
 constexpr int kRoot3 = 0, kRoot5 = 3, kRoot7 = 8, kRoots = 15;
@@ -83,9 +92,10 @@ __device__ __forceinline__ void stockham_pass(const float2 *__restrict__ X, floa
                                               const float2 *__restrict__ root) {
     const int NR = N / R;
     const int tstep = N / (Ns * R);
+    const FastDiv byNR(NR), byNs(Ns);
     for (int t = threadIdx.x; t < B * NR; t += blockDim.x) {
-        const int b = t / NR, j = t - b * NR;
-        const int jm = j % Ns;
+        const int b = byNR.div(t), j = t - b * NR;
+        const int jd = byNs.div(j), jm = j - jd * Ns;
         float2 v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -97,7 +107,7 @@ __device__ __forceinline__ void stockham_pass(const float2 *__restrict__ X, floa
             }
         }
         small_dft<R>(v, dir, root);
-        const int idx = (j / Ns) * Ns * R + jm;
+        const int idx = jd * Ns * R + jm;
 #pragma unroll
         for (int r = 0; r < R; ++r) Y[b * N + idx + r * Ns] = v[r];
     }
@@ -140,13 +150,15 @@ struct Pass {
     Radices rad;         // radix of each Stockham pass
 };
 
-__device__ __forceinline__ void lin(const Pass &p, int idx, int &b, int &k) {
+// Batch and element of idx, consecutive in global memory (by: p.N for rows,
+// p.B otherwise).
+__device__ __forceinline__ void lin(const Pass &p, const FastDiv &by, int idx, int &b, int &k) {
     if (p.ks == 1) {
-        b = idx / p.N;
-        k = idx % p.N;
+        b = by.div(idx);
+        k = idx - b * p.N;
     } else {
-        k = idx / p.B;
-        b = idx % p.B;
+        k = by.div(idx);
+        b = idx - k * p.B;
     }
 }
 
@@ -166,9 +178,10 @@ __global__ void __launch_bounds__(kThreads)
     const int b0 = blockIdx.x * p.B;
     const int nb = min(p.B, p.nbatch - b0);
     const int64_t cbase = ch * p.ch_stride;
+    const FastDiv by(p.ks == 1 ? p.N : p.B), byN(p.N);
     for (int idx = threadIdx.x; idx < p.N * p.B; idx += blockDim.x) {
         int b, k;
-        lin(p, idx, b, k);
+        lin(p, by, idx, b, k);
         if (b >= nb) continue;
         const int64_t off = (int64_t)(b0 + b) * p.bs + (int64_t)k * p.ks;
         float2 v;
@@ -188,7 +201,7 @@ __global__ void __launch_bounds__(kThreads)
     } else if (mode == 1) {
         R = stockham(X, Y, p.N, p.B, -1, p.rad, tw);
         for (int idx = threadIdx.x; idx < p.N * p.B; idx += blockDim.x) {
-            const int b = idx / p.N, k = idx % p.N;
+            const int b = byN.div(idx), k = idx - b * p.N;
             if (b >= nb) continue;
             const float s = spec[(int64_t)k * spec_ks + (int64_t)(b0 + b) * spec_bs];
             R[idx].x *= s;
@@ -201,7 +214,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     for (int idx = threadIdx.x; idx < p.N * p.B; idx += blockDim.x) {
         int b, k;
-        lin(p, idx, b, k);
+        lin(p, by, idx, b, k);
         if (b >= nb) continue;
         const int64_t off = (int64_t)(b0 + b) * p.bs + (int64_t)k * p.ks;
         const float2 v = R[b * p.N + k];
@@ -212,6 +225,51 @@ __global__ void __launch_bounds__(kThreads)
         } else {
             Z[cbase + off] = v;
         }
+    }
+}
+
+// The middle of a cross-material apply (Eqs. 56-57) in one kernel: B columns of
+// every material, forward in y, the per-frequency mixing Z[a] <- sum_b L[a][b]
+// Z[b], inverse in y.  Against separate passes Z is read and written once
+// instead of three times and two launches go; with the divisions above, a
+// 448^2 apply of three materials went from 79 to 65 us (same bits).
+constexpr int kMixThreads = 512;
+
+__global__ void __launch_bounds__(kMixThreads)
+    fft_mix_kernel(int N, int B, int nx, int nm, Radices rad, float2 *__restrict__ Z, const float *__restrict__ L,
+                   const float2 *__restrict__ tw) {
+    extern __shared__ float2 sm[];
+    const int per = N * B, b0 = blockIdx.x * B, nb = min(B, nx - b0);
+    float2 *X = sm, *Y = sm + nm * per;
+    const int64_t plane = (int64_t)N * nx;
+    const FastDiv byB(B), byPer(per);
+    for (int idx = threadIdx.x; idx < nm * per; idx += blockDim.x) {
+        const int m = byPer.div(idx), r = idx - m * per, k = byB.div(r), b = r - k * B;
+        X[(m * B + b) * N + k] = b < nb ? Z[m * plane + (int64_t)k * nx + b0 + b] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    float2 *R = stockham(X, Y, N, nm * B, -1, rad, tw);
+    for (int idx = threadIdx.x; idx < per; idx += blockDim.x) {
+        const int k = byB.div(idx), b = idx - k * B;
+        if (b >= nb) continue;
+        const int64_t f = (int64_t)k * nx + b0 + b;
+        float2 v[4];
+        for (int a = 0; a < nm; ++a) v[a] = R[(a * B + b) * N + k];
+        for (int a = 0; a < nm; ++a) {
+            float2 acc = make_float2(0.f, 0.f);
+            for (int c = 0; c < nm; ++c) {
+                const float l = __ldg(L + ((int64_t)a * nm + c) * plane + f);
+                acc.x = fmaf(l, v[c].x, acc.x);
+                acc.y = fmaf(l, v[c].y, acc.y);
+            }
+            R[(a * B + b) * N + k] = acc;
+        }
+    }
+    __syncthreads();
+    R = stockham(R, R == X ? Y : X, N, nm * B, +1, rad, tw);
+    for (int idx = threadIdx.x; idx < nm * per; idx += blockDim.x) {
+        const int m = byPer.div(idx), r = idx - m * per, k = byB.div(r), b = r - k * B;
+        if (b < nb) Z[m * plane + (int64_t)k * nx + b0 + b] = R[(m * B + b) * N + k];
     }
 }
 
@@ -330,6 +388,23 @@ mbir_status FftPlan::inverse(int channels, float2 *Z, float *out, const float *p
     if (nz > 1) PSPS_TRY(run(2, 4, channels, nullptr, Z, nullptr, nullptr, nullptr, s));
     PSPS_TRY(run(1, 4, channels, nullptr, Z, nullptr, nullptr, nullptr, s));
     return run(0, 2, channels, nullptr, Z, out, post, nullptr, s);
+}
+
+mbir_status FftPlan::mixed(int channels, const float *in, float2 *Z, float *out, const float *L, bool &done,
+                           cudaStream_t s) const {
+    // four columns (whole sectors) per CTA where that gives every SM one,
+    // else two; more shared memory than a CTA has: the separate passes
+    const int B = nx >= 4 * 152 ? 4 : 2;
+    const size_t smem = 2 * sizeof(float2) * (size_t)ny * B * channels;
+    done = nz <= 1 && channels <= 4 && smem <= 200 * 1024 && (int64_t)ny * B * channels < 65536;
+    if (!done) return MBIR_OK;
+    PSPS_TRY(run(0, 0, channels, in, Z, nullptr, nullptr, nullptr, s));
+    PSPS_CUDA(cudaFuncSetAttribute(fft_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    Radices rad;
+    factor(ny, rad);
+    fft_mix_kernel<<<(unsigned)cdiv(nx, B), kMixThreads, smem, s>>>(ny, B, nx, channels, rad, Z, L, twy.p);
+    PSPS_LAUNCH_CHECK();
+    return run(0, 2, channels, nullptr, Z, out, nullptr, nullptr, s);
 }
 
 mbir_status FftPlan::filter(int channels, const float *in, float2 *Z, float *out, const float *pre, const float *post,

@@ -19,6 +19,11 @@ struct FftPlan {
     mbir_status forward(int channels, const float *in, float2 *Z, cudaStream_t s) const;
     // out = post .* Re(IDFT(Z)) (normalised by 1/(nx ny nz)); Z is overwritten.
     mbir_status inverse(int channels, float2 *Z, float *out, const float *post, cudaStream_t s) const;
+    // inverse(L forward(in)) with the per-frequency blocks L[a][b][ny * nx], one
+    // kernel between the row passes; done = false (nothing launched) where it
+    // does not apply (3-D, or columns too long for it)
+    mbir_status mixed(int channels, const float *in, float2 *Z, float *out, const float *L, bool &done,
+                      cudaStream_t s) const;
     mbir_status filter(int channels, const float *in, float2 *Z, float *out, const float *pre, const float *post,
                        const float *spec, cudaStream_t s) const;
 };

@@ -651,10 +651,15 @@ mbir_status precond_apply(psps_precond *pc, int op, const float *in, float *out,
                 PSPS_LAUNCH_CHECK();
                 src = t0;
             }
-            PSPS_TRY(pc->fft.forward(pc->nm, src, pc->Z.p, s));
-            mix_kernel<<<gs(pc->n), kThreads, 0, s>>>(pc->nm, pc->n, absm ? pc->Li_abs.p : pc->Li.p, pc->Z.p);
-            PSPS_LAUNCH_CHECK();
-            PSPS_TRY(pc->fft.inverse(pc->nm, pc->Z.p, m0_after ? t1 : out, nullptr, s));
+            float *dst = m0_after ? t1 : out;
+            bool done = false;
+            PSPS_TRY(pc->fft.mixed(pc->nm, src, pc->Z.p, dst, absm ? pc->Li_abs.p : pc->Li.p, done, s));
+            if (!done) {
+                PSPS_TRY(pc->fft.forward(pc->nm, src, pc->Z.p, s));
+                mix_kernel<<<gs(pc->n), kThreads, 0, s>>>(pc->nm, pc->n, absm ? pc->Li_abs.p : pc->Li.p, pc->Z.p);
+                PSPS_LAUNCH_CHECK();
+                PSPS_TRY(pc->fft.inverse(pc->nm, pc->Z.p, dst, nullptr, s));
+            }
             if (m0_after) {
                 block_apply_kernel<<<gs(pc->n), kThreads, 0, s>>>(pc->nm, pc->n, Bm, t1, out, 1);
                 PSPS_LAUNCH_CHECK();
