@@ -112,7 +112,7 @@ __global__ void cone_pack_z_kernel(const float *__restrict__ x, int nm, int P, i
 // 8-column group writes whole 32-byte sectors.
 // Bound by L1 latency and issue.  Two materials, 256^3 from 360 x 384 x 512
 // rays: 12.6 ms (29.2 ms with one thread per ray along the detector rows,
-// whose four taps touched 10.8 sectors per request against 4.9 here); 128^3
+// whose four taps touched 10.8 sectors per request against 6.2 here); 128^3
 // from 180 x 192 x 256: 0.85 ms (1.80).  Tried: one register set (15.1 ms,
 // long-scoreboard stalls), the plane's lines staged in shared memory by 16-byte
 // asynchronous copies (22 ms: a third more instructions and a barrier per

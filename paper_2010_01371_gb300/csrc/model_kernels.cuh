@@ -33,13 +33,14 @@ __device__ __forceinline__ float transmission(float z) { return exp2f(z * -1.442
 // load brings two of them, for both rays): q_m = -log2(e) Q[E][m] (the sum
 // over m is then the exponent of 2; factors of log2 e leave per ray), then
 // S[c][E].
-// Measured on 720 x 888 rays, 2 materials, 121 energies, 2 channels: numerators
-// 96 -> 75 us, line-search evaluation 58 -> 48 us, the eight halving
-// candidates 140 -> 90 us against one ray per thread with exp2f's subnormal
-// handling and every channel at every energy; with blur and correlated noise
-// the data-term gradient 171 -> 98 us.  The FP32 pipe is half busy (26 of 46
-// cycles per energy, pair of rays and scheduler) and so is issue; more rays
-// (x 8) run at the same rate.
+// Measured on 720 x 888 rays, 2 materials, 121 energies, 2 channels (ncu, cold):
+// numerators 117 -> 80 us, line-search evaluation 76 -> 55 us, the eight halving
+// candidates 181 -> 107 us against one ray per thread with exp2f's subnormal
+// handling and every channel at every energy; 3 materials, 4 channels: model
+// stage 146 -> 85 us, line search 395 -> 231 us per iteration; with blur and
+// correlated noise the data-term gradient 174 -> 96 us.  The FP32 pipe is half
+// busy and so is issue (50 % each for the evaluation); more rays (x 8) run at
+// the same rate.
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLog2eHi = (float)1.4426950408889634;                            // log2(e) = hi + lo
 constexpr float kLog2eLo = (float)(1.4426950408889634 - (double)(float)1.4426950408889634);
