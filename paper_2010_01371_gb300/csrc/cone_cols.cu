@@ -375,17 +375,25 @@ struct ColDesc {                 // of (column q / kP, plane q % kP) of the curr
     float2 k[32];                // row spacing on the plane (0: no voxel reached), 1 / spacing on the middle plane
 };
 
-// One column: NR rows from the one nearest (z's row) - first on, on the
-// patch's kP planes.  src: row 0 of the column.
-template <int A, int C, int NR>
+// One column: NR rows on the patch's kP planes, row `skip` of the window that
+// starts at the row nearest (z's row) - first being the first of them.  The
+// window's start is rounded once per z and column, whatever the pass: starts
+// rounded pass by pass need not be whole passes apart (FP32 values of
+// different binades), which lost or doubled a row at the seam.  src: row 0 of
+// the column; wide: rows of the window before the last pass (0: one pass).
+template <int A, int C, int NR, bool MULTI>
 __device__ __forceinline__ void cols_column(const float *__restrict__ src, const float2 *dk, const float4 *da,
-                                            const float4 *db, float mz, float rc, float first, int n_v,
-                                            f32x2 (&acc)[kP][kP][C / 2]) {
+                                            const float4 *db, float mz, float rc, float first, int skip, int wide,
+                                            int n_v, f32x2 (&acc)[kP][kP][C / 2]) {
     float fr = fmaf(-mz, dk[0].y, rc - first);
-    fr = fminf(fmaxf(fr, (float)-NR), (float)n_v);
+    fr = fminf(fmaxf(fr, (float)-(NR + wide)), (float)n_v);
     const float rn = fr + kSplitMagic;
-    const int r0 = __float_as_int(rn) - __float_as_int(kSplitMagic);
-    const float w0 = (rn - kSplitMagic) - rc;
+    int r0 = __float_as_int(rn) - __float_as_int(kSplitMagic);
+    float w0 = (rn - kSplitMagic) - rc;
+    if constexpr (MULTI) {
+        r0 = min(max(r0 + skip, -NR), n_v);   // a pass wholly outside reads zero rows
+        w0 = (float)r0 - rc;
+    }
     src += r0 * C;
     f32x2 s[NR][C / 2];
 #pragma unroll
@@ -431,11 +439,11 @@ __device__ __forceinline__ void cols_column(const float *__restrict__ src, const
     }
 }
 
-template <int A, int C, int NR>
+template <int A, int C, int NR, bool MULTI>
 __device__ __forceinline__ void cols_gather(const mbir_geometry &g, const float4 *__restrict__ cv,
                                             const float2 *__restrict__ wv, const float *__restrict__ wsv, int ua, int ub,
-                                            bool mixed, int x0, int y0, float mz, float zmax, float first, ColDesc &desc,
-                                            f32x2 (&acc)[kP][kP][C / 2]) {
+                                            bool mixed, int x0, int y0, float mz, float zmax, float first, int skip,
+                                            int wide, ColDesc &desc, f32x2 (&acc)[kP][kP][C / 2]) {
     static_assert(kP == 4, "a lane per (column, plane) pair of eight columns, four weights per descriptor");
     const int na = A == 0 ? g.nx : g.ny, nb = A == 0 ? g.ny : g.nx;
     const int a0 = A == 0 ? x0 : y0, b0 = (A == 0 ? y0 : x0) - (nb >> 1);
@@ -474,9 +482,11 @@ __device__ __forceinline__ void cols_gather(const mbir_geometry &g, const float4
         for (int c = 0; c < nu; ++c) {
             const float *src = wsv + ((int64_t)(ug + c) * stride + kRowPad) * C;
             if (NR == 4 && (few >> (c * kP) & 15u) == 15u)
-                cols_column<A, C, 3>(src, &desc.k[c * kP], &desc.wa[c * kP], &desc.wb[c * kP], mz, rc, 1.f, n_v, acc);
+                cols_column<A, C, 3, false>(src, &desc.k[c * kP], &desc.wa[c * kP], &desc.wb[c * kP], mz, rc, 1.f, 0, 0, n_v,
+                                            acc);
             else
-                cols_column<A, C, NR>(src, &desc.k[c * kP], &desc.wa[c * kP], &desc.wb[c * kP], mz, rc, first, n_v, acc);
+                cols_column<A, C, NR, MULTI>(src, &desc.k[c * kP], &desc.wa[c * kP], &desc.wb[c * kP], mz, rc, first, skip,
+                                             wide, n_v, acc);
         }
     }
 }
@@ -531,11 +541,14 @@ __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
             const int64_t cv = (int64_t)(vb + q) * g.n_u;
             const float *wsv = ws + (int64_t)(vb + q) * vstride;
             for (int r = 0; r < (MULTI ? nrows : 1); r += NR) {
-                const float first = MULTI ? 0.5f * (nrows - 1) - (float)r : 0.5f * (NR - 1);
+                const float first = 0.5f * ((MULTI ? nrows : NR) - 1);
+                const int wide = MULTI ? nrows - NR : 0;
                 if (ax & 1)
-                    cols_gather<0, C, NR>(g, col + cv, colw + cv, wsv, xa, xb, ax == 3, x0, y0, mz, zmax, first, desc, acc);
+                    cols_gather<0, C, NR, MULTI>(g, col + cv, colw + cv, wsv, xa, xb, ax == 3, x0, y0, mz, zmax, first, r,
+                                                 wide, desc, acc);
                 if (ax & 2)
-                    cols_gather<1, C, NR>(g, col + cv, colw + cv, wsv, ya, yb, ax == 3, x0, y0, mz, zmax, first, desc, acc);
+                    cols_gather<1, C, NR, MULTI>(g, col + cv, colw + cv, wsv, ya, yb, ax == 3, x0, y0, mz, zmax, first, r,
+                                                 wide, desc, acc);
             }
         }
 #pragma unroll
