@@ -119,8 +119,8 @@ mbir_status mbir_backproject(mbir_plan *plan, const float *s, float *x, int n_ma
  * bitwise reproducible.  A non-finite input makes its channel's image NaN.
  * It needs 8 bytes x n_mat_max x n_pix of plan scratch.  3-D (cone): 0 =
  * voxel-driven over detector columns (default: the in-plane weights and the
- * row spacing of a column are common to its rays; FP32 sums over at most 32
- * views, added in a fixed order, so bitwise reproducible; a non-finite input
+ * row spacing of a column are common to its rays; FP32 sums over eight views,
+ * added with compensation in a fixed order, so bitwise reproducible; a non-finite input
  * makes its channel's image NaN).  Plans with rays that the z axis drives, with
  * more than 48 detector rows per voxel layer's reach or with the source within
  * four voxels of the volume's radius run a tile scatter instead: a CTA per

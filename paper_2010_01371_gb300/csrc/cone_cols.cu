@@ -354,18 +354,28 @@ __device__ __forceinline__ int2 patch_columns(const mbir_geometry &g, float4 V, 
 // eight columns at a time, and read back from shared memory as broadcasts;
 // all kP weights are applied (most are zero), which costs less than branching
 // to the two that are not.  The accumulators stay in registers and there are
-// no atomics.  FP32 sums run over at most 32 views and are then added to the
-// thread's totals in shared memory; the image is written once, or, when the
-// views are split over blockIdx.y so that a small volume fills the GPU, as one
-// partial image per split that cols_reduce_kernel adds in a fixed order.
+// no atomics.  FP32 sums run over kGroup views and are then added to the
+// thread's totals in shared memory, with the rounding of every such add kept
+// and put back in the next (a compensation of 8 significant bits below the
+// total's 24, so the totals still leave room for 16 warps per SM; 32-bit
+// compensations leave room for 12 and take 28.2 ms where this takes 23.9).
+// The image is written once, or, when the views are split over blockIdx.y so
+// that a small volume fills the GPU, as one partial image per split that
+// cols_reduce_kernel adds in a fixed order.
 // Either way the result does not depend on the order in which the CTAs run.
+// Why so exact: the cross-material Fourier and wavelet preconditioners
+// difference two materials' gradients after a spatial filter.  Relative error
+// of the filtered gradient near convergence, 128^3, 180 / 720 views: plain
+// totals of 32-view sums 7.7e-6 / 16.6e-6, this 4.8e-6 / 10.2e-6 (kGroup = 16:
+// 5.5e-6 / 11.0e-6), the tile scatter with low words 5.8e-6 / 11.5e-6.
 // Channel pairs use the packed operations.
 // Bound by the shared-memory / L1 pipe (64 % busy, mostly the row loads: 16
 // sectors each) and the latency its 16 warps per SM leave exposed.  Four
-// channels, 256^3 from 360 x 384 x 512 rays: 22.4 ms with the weighting pass
-// (77.7 ms for the ray-driven tile scatter); 128^3 from 180 x 192 x 256: 1.66 ms
-// (5.3).  Two channels: 15.7 and 1.14 ms.  A branch to the two voxels with
-// nonzero weight instead of all four weights took 29 ms at 256^3, CTAs of 8
+// channels, 256^3 from 360 x 384 x 512 rays: 23.9 ms with the weighting pass
+// (77.7 ms for the ray-driven tile scatter); 128^3 from 180 x 192 x 256: 1.77 ms
+// (5.3).  Two channels: 16.2 and 1.17 ms.  The compensated totals are 6 % of
+// the four-channel times.  With plain totals, a branch to the two voxels with
+// nonzero weight instead of all four weights took 29 ms (22.4) at 256^3, CTAs of 8
 // and 16 warps, planes tested in pairs and an L1 prefetch of the next view's
 // rows were no faster.
 constexpr int kBX = 2, kBY = 2, kBWarps = kBX * kBY;   // warps per CTA: kBX x kBY patches of the same 32 z
@@ -491,6 +501,21 @@ __device__ __forceinline__ void cols_gather(const mbir_geometry &g, const float4
     }
 }
 
+constexpr int kGroup = 8;   // views per compensated add
+static_assert(32 % kGroup == 0, "groups end with the views that a warp's lanes look up together");
+
+// Compensations of a pair of totals, each rounded to its upper 16 bits.
+__device__ __forceinline__ f32x2 unpack_low(unsigned v) {
+    return pair2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+__device__ __forceinline__ unsigned pack_low(f32x2 v) {
+    float a, b;
+    unpair2(v, a, b);
+    unsigned d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    return d;
+}
+
 // MULTI: the rows that reach one z exceed NR, so several passes of NR.
 template <int C, int NR, bool MULTI>
 __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
@@ -501,7 +526,8 @@ __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
     constexpr int N = kP * kP * C;
     extern __shared__ float4 back_smem[];
     ColDesc *descs = reinterpret_cast<ColDesc *>(back_smem);
-    float(*tot)[32 * kBWarps] = reinterpret_cast<float(*)[32 * kBWarps]>(descs + kBWarps);
+    f32x2(*tot)[32 * kBWarps] = reinterpret_cast<f32x2(*)[32 * kBWarps]>(descs + kBWarps);
+    unsigned(*low)[32 * kBWarps] = reinterpret_cast<unsigned(*)[32 * kBWarps]>(tot + N / 2);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // CTA (xt, yt, zt), x fastest
     const int nxt = (g.nx + kBX * kP - 1) / (kBX * kP), nyt = (g.ny + kBY * kP - 1) / (kBY * kP);
@@ -515,15 +541,15 @@ __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
     const int vbeg = blockIdx.y * vchunk, vend = min(vbeg + vchunk, g.n_views);
     const int64_t vstride = (int64_t)g.n_u * (g.n_v + 2 * kRowPad) * C;
 #pragma unroll
-    for (int q = 0; q < N; ++q) tot[q][threadIdx.x] = 0.f;
+    for (int q = 0; q < N / 2; ++q) tot[q][threadIdx.x] = 0ull, low[q][threadIdx.x] = 0u;
+    f32x2 acc[kP][kP][C / 2];
+#pragma unroll
+    for (int a = 0; a < kP; ++a)
+#pragma unroll
+        for (int b = 0; b < kP; ++b)
+#pragma unroll
+            for (int c = 0; c < C / 2; ++c) acc[a][b][c] = 0ull;
     for (int vb = vbeg; vb < vend; vb += 32) {
-        f32x2 acc[kP][kP][C / 2];
-#pragma unroll
-        for (int a = 0; a < kP; ++a)
-#pragma unroll
-            for (int b = 0; b < kP; ++b)
-#pragma unroll
-                for (int c = 0; c < C / 2; ++c) acc[a][b][c] = 0ull;
         // lane q: the patch's columns in view vb + q, per driving axis
         int axes = 0;
         int2 ux = make_int2(0, -1), uy = make_int2(0, -1);
@@ -550,18 +576,21 @@ __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
                     cols_gather<1, C, NR, MULTI>(g, col + cv, colw + cv, wsv, ya, yb, ax == 3, x0, y0, mz, zmax, first, r,
                                                  wide, desc, acc);
             }
+            if ((q + 1) % kGroup && q + 1 < nv) continue;
+#pragma unroll
+            for (int a = 0; a < kP; ++a)
+#pragma unroll
+                for (int b = 0; b < kP; ++b)
+#pragma unroll
+                    for (int h = 0; h < C / 2; ++h) {
+                        const int k = (a * kP + b) * (C / 2) + h;
+                        const f32x2 t0 = tot[k][threadIdx.x];
+                        const f32x2 yk = sub2(acc[a][b][h], unpack_low(low[k][threadIdx.x])), t1 = add2(t0, yk);
+                        low[k][threadIdx.x] = pack_low(sub2(sub2(t1, t0), yk));
+                        tot[k][threadIdx.x] = t1;
+                        acc[a][b][h] = 0ull;
+                    }
         }
-#pragma unroll
-        for (int a = 0; a < kP; ++a)
-#pragma unroll
-            for (int b = 0; b < kP; ++b)
-#pragma unroll
-                for (int h = 0; h < C / 2; ++h) {
-                    float lo, hi;
-                    unpair2(acc[a][b][h], lo, hi);
-                    tot[(a * kP + b) * C + 2 * h][threadIdx.x] += lo;
-                    tot[(a * kP + b) * C + 2 * h + 1][threadIdx.x] += hi;
-                }
     }
     if (z >= g.nz) return;
     const int64_t npix = (int64_t)g.nx * g.ny * g.nz;
@@ -569,7 +598,9 @@ __global__ void __launch_bounds__(32 * kBWarps, C == 4 ? 4 : 5)
         const bool bad = !(__uint_as_float(__ldg(smax + c)) <= 3.0e38f);   // a NaN or infinity poisons its channel
         for (int b = 0; b < kP && y0 + b < g.ny; ++b)
             for (int a = 0; a < kP && x0 + a < g.nx; ++a) {
-                const float v = bad ? __int_as_float(0x7fc00000) : tot[(a * kP + b) * C + c][threadIdx.x];
+                float t[2];
+                unpair2(tot[((a * kP + b) * C + c) / 2][threadIdx.x], t[0], t[1]);
+                const float v = bad ? __int_as_float(0x7fc00000) : (c & 1 ? t[1] : t[0]);
                 const int64_t o = (int64_t)c * npix + ((int64_t)z * g.ny + y0 + b) * g.nx + x0 + a;
                 if (part_stride)
                     x[blockIdx.y * part_stride + o] = v;
@@ -698,7 +729,7 @@ mbir_status backproject_cols(mbir_plan *p, const float *sino, float *x, int nc, 
     float *dst = ns > 1 ? p->col_part.p : x;
     const int64_t stride = ns > 1 ? (int64_t)4 * p->n_pix : 0;
     auto run = [&](auto nr, auto multi) {
-        constexpr size_t smem = kBWarps * (sizeof(ColDesc) + sizeof(float) * kP * kP * C * 32);
+        constexpr size_t smem = kBWarps * (sizeof(ColDesc) + (sizeof(f32x2) + sizeof(unsigned)) * (kP * kP * C / 2) * 32);
         cudaFuncSetAttribute(back_cols_kernel<C, decltype(nr)::value, decltype(multi)::value>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         back_cols_kernel<C, decltype(nr)::value, decltype(multi)::value><<<grd, 32 * kBWarps, smem, s>>>(
