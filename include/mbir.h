@@ -122,8 +122,9 @@ mbir_status mbir_backproject(mbir_plan *plan, const float *s, float *x, int n_ma
  * row spacing of a column are common to its rays; FP32 sums over eight views,
  * added with compensation in a fixed order, so bitwise reproducible; a non-finite input
  * makes its channel's image NaN).  Plans with rays that the z axis drives, with
- * more than 48 detector rows per voxel layer's reach or with the source within
- * four voxels of the volume's radius run a tile scatter instead: a CTA per
+ * more than 48 detector rows per voxel layer's reach, with the source within
+ * four voxels of the volume's radius, or with fewer than 12 rows or layers
+ * (fewer still for images up to 128 x 128) run a tile scatter instead: a CTA per
  * 8 x 8 x 16-voxel tile runs over every
  * view, stages the rays of the tile's detector box and adds each (ray, tile
  * plane) sample's bilinear terms to 32-bit fixed-point shared-memory
@@ -183,7 +184,7 @@ mbir_status mbir_plan_tuning(const mbir_plan *plan, int *fwd_mode, int *strip_bi
  * shared-memory strips of the image, every lane on the same driving index
  * (deterministic).  Cone beam: one algorithm whatever the mode (a warp per
  * detector column, lanes on its rows; one thread per ray for plans with rays
- * that the z axis drives).  All use the same per-ray Joseph weights.
+ * that the z axis drives or with few rows that meet the volume).  All use the same per-ray Joseph weights.
  * MBIR_ERR_ARG for other modes. */
 mbir_status mbir_plan_set_projector(mbir_plan *plan, int mode);
 

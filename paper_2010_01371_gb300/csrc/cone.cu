@@ -12,10 +12,12 @@
 // on plane i its height is z = (row offset) k(i) with k(i) = q0 + (i - c_a) dq
 // common to the column.  These four numbers per column are set up in FP64 once
 // per plan (cone_cols.cuh); cone_cols.cu holds the forward and the transpose
-// built on them, which every plan without z-driven rays uses.
+// built on them, which plans without z-driven rays use unless their rows or
+// layers are few (cone_cols_forward, cone_cols_setup).
 //
 // This file holds the set-up and the general kernels: plans with z-driven rays
-// (detector half-height above sdd / sqrt 2) and the alternative transposes.
+// (detector half-height above sdd / sqrt 2) or few rows and the alternative
+// transposes.
 // They read a per-ray table (24 bytes per ray) derived from the column
 // constants: coordinates relative to the middle of the volume (index n / 2
 // of the interpolated axis, less 1/2 for the conversion-free sample split),
@@ -183,11 +185,15 @@ __device__ __forceinline__ void decode3(float2 b, int &axis, int &lo, int &hi) {
     hi = (bits >> 17) & 0x7fff;
 }
 
-// One thread per ray, each over its own range; two samples' tap loads are
-// issued before use.  Copies of the volume as cone_cols.cuh describes; a
-// sample's lower tap indices are clamped to [-kPad, n + kPad - 2]: a sample the
-// clamp moves lies wholly outside the volume (its taps are at <= -2 or >= n),
-// and the clamped taps then read border zeros, as the true ones are.
+// One thread per ray (plans with z-driven rays, or too few rows for a warp per
+// detector column: cone_cols_forward), neighbouring threads on neighbouring
+// detector columns, each over its own range; two samples' tap loads are issued
+// before use.  With the copies ordered along z, as the columns read them, this
+// kernel's lanes touch one line each: 4.2 ms instead of 2.0 for 256 x 256 x 32
+// voxels from 360 x 32 x 512 rays, 6.2 instead of 2.8 for two materials.
+// A sample's lower tap indices are clamped to [-kPad, n + kPad - 2]: a sample
+// the clamp moves lies wholly outside the volume (its taps are at <= -2 or
+// >= n), and the clamped taps then read border zeros, as the true ones are.
 template <int NM>
 __global__ void __launch_bounds__(kThreads)
     fwd_cone_kernel(mbir_geometry g, const float4 *__restrict__ ta, const float2 *__restrict__ tb,
@@ -200,37 +206,40 @@ __global__ void __launch_bounds__(kThreads)
     int axis, lo, hi;
     decode3(B, axis, lo, hi);
     using T = typename CPack<NM>::T;
-    const T *src = axis == 0 ? ox : (axis == 1 ? oy : oz);
     const int nb = axis == 0 ? g.ny : g.nx, nc = axis == 2 ? g.ny : g.nz;
     const int nbp = nb + 2 * kPad, ncp = nc + 2 * kPad, cb = nb >> 1, cc = nc >> 1;
+    const T *src = axis == 0 ? ox : (axis == 1 ? oy : oz);
     const float ca = 0.5f * ((axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nz)) - 1);
     float acc[NM], comp[NM];
 #pragma unroll
     for (int m = 0; m < NM; ++m) acc[m] = comp[m] = 0.f;
-    for (int i = lo; i <= hi; i += 2) {
+    // (written out rather than shared between pairs and the last sample: a
+    // lambda for either half, or coordinates kept relative to the middle, cost
+    // 10-20 % with two and four materials)
+    int i = lo;
+    for (; i + 1 <= hi; i += 2) {
         T v[2][4];
         float gb[2], gc[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int iu = min(i + u, hi);
-            const float t = (float)iu - ca;
+            const float t = (float)(i + u) - ca;
             const int ib0 = joseph_split(fmaf(t, A.y, A.x), gb[u]) + cb, ic0 = joseph_split(fmaf(t, A.w, A.z), gc[u]) + cc;
             const int ibc = min(max(ib0, -kPad), nb + kPad - 2), icc = min(max(ic0, -kPad), nc + kPad - 2);
-            const T *tap = src + ((int64_t)iu * nbp + ibc + kPad) * ncp + icc + kPad;
+            const T *tap = src + ((int64_t)(i + u) * ncp + icc + kPad) * nbp + ibc + kPad;
             v[u][0] = __ldg(tap);
             v[u][1] = __ldg(tap + 1);
-            v[u][2] = __ldg(tap + ncp);
-            v[u][3] = __ldg(tap + ncp + 1);
+            v[u][2] = __ldg(tap + nbp);
+            v[u][3] = __ldg(tap + nbp + 1);
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            if (i + u > hi) break;
             float sm[NM];
 #pragma unroll
             for (int m = 0; m < NM; ++m) sm[m] = 0.f;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float wbc = ((q >> 1) ? gb[u] : 1.f - gb[u]) * ((q & 1) ? gc[u] : 1.f - gc[u]);
+                const float wc = (q >> 1) ? gc[u] : 1.f - gc[u];
+                const float wbc = ((q & 1) ? gb[u] : 1.f - gb[u]) * wc;
                 float val[NM];
                 CPack<NM>::get(v[u][q], val);
 #pragma unroll
@@ -243,6 +252,34 @@ __global__ void __launch_bounds__(kThreads)
                 comp[m] = __fsub_rn(__fsub_rn(tt, acc[m]), yk);
                 acc[m] = tt;
             }
+        }
+    }
+    for (; i <= hi; ++i) {
+        const float t = (float)i - ca;
+        float gb, gc, sm[NM];
+        const int ib0 = joseph_split(fmaf(t, A.y, A.x), gb) + cb, ic0 = joseph_split(fmaf(t, A.w, A.z), gc) + cc;
+        const int ibc = min(max(ib0, -kPad), nb + kPad - 2), icc = min(max(ic0, -kPad), nc + kPad - 2);
+        const T *tap = src + ((int64_t)i * ncp + icc + kPad) * nbp + ibc + kPad;
+#pragma unroll
+        for (int m = 0; m < NM; ++m) sm[m] = 0.f;
+#pragma unroll
+        for (int jc = 0; jc < 2; ++jc) {
+            const float wc = jc ? gc : 1.f - gc;
+#pragma unroll
+            for (int jb = 0; jb < 2; ++jb) {
+                const float wbc = (jb ? gb : 1.f - gb) * wc;
+                float val[NM];
+                CPack<NM>::get(__ldg(tap + jc * nbp + jb), val);
+#pragma unroll
+                for (int m = 0; m < NM; ++m) sm[m] = fmaf(wbc, val[m], sm[m]);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const float yk = __fsub_rn(sm[m], comp[m]);
+            const float tt = __fadd_rn(acc[m], yk);
+            comp[m] = __fsub_rn(__fsub_rn(tt, acc[m]), yk);
+            acc[m] = tt;
         }
     }
 #pragma unroll
@@ -1009,7 +1046,6 @@ mbir_status cone_setup(mbir_plan *p) {
     PSPS_TRY(p->ray3b.alloc(p->n_rays));
     PSPS_TRY(p->view_axes.alloc(p->g.n_views));
     PSPS_TRY(p->view_axes.zero(0));
-    PSPS_TRY(p->wsino.alloc((size_t)4 * p->g.n_views * p->g.n_u * (p->g.n_v + 2 * kRowPad)));
     PSPS_TRY(p->wmax.alloc(4));
     {
         // Rays of one view that reach one voxel j (any driving axis), for the
@@ -1052,6 +1088,10 @@ mbir_status cone_setup(mbir_plan *p) {
     setup_rays3d_kernel<<<grd, kThreads>>>(p->g, p->view.p, p->col.p, p->colw.p, p->ray.p, p->ray3b.p, p->view_axes.p);
     PSPS_LAUNCH_CHECK();
     PSPS_TRY(cone_cols_setup(p));
+    // up to four channels of a weighted sinogram; the column transpose wants
+    // zero rows around every detector column
+    const int64_t rows = p->g.n_v + (p->col_rows > 0 ? 2 * kRowPad : 0);
+    PSPS_TRY(p->wsino.alloc((size_t)(4 * n_cols * rows)));
     // the copy of the z-driven rays, only where there are such rays
     return p->cols ? MBIR_OK : p->xcol3.alloc(cone_pack_floats(p->g));
 }
@@ -1062,12 +1102,12 @@ mbir_status project_cone(mbir_plan *p, const float *x, float *l, int n_mat, cuda
         const int nm = n_mat - m0 < 4 ? n_mat - m0 : 4;
         const float *xm = x + (int64_t)m0 * p->n_pix;
         float *lm = l + (int64_t)m0 * p->n_rays;
-        if (p->cols) {
+        const int P = nm == 1 ? 1 : (nm == 2 ? 2 : 4);
+        if (p->cols && cone_cols_forward(g, P)) {
             PSPS_TRY(project_cone_cols(p, xm, lm, nm, s));
             continue;
         }
-        const int P = nm == 1 ? 1 : (nm == 2 ? 2 : 4);
-        PSPS_TRY(cone_pack(p, xm, nm, P, true, s));
+        PSPS_TRY(cone_pack_rows(p, xm, nm, P, !p->cols, s));
         const float *ox = p->xcol.p, *oy = p->xrow.p, *oz = p->xcol3.p;
         const unsigned gr = (unsigned)cdiv(p->n_rays, kThreads);
         if (P == 1)

@@ -19,31 +19,33 @@ constexpr int kThreads = 256;
 // ------------------------------------------------------------------ packing
 
 // Border cells of the copies (kPad cells on every side of b and c), P floats
-// each: per plane, 2 kPad full lines along c and n_b segments of 2 kPad cells.
-__global__ void cone_border_kernel(int P, int nx, int ny, int nz, int copies, float *__restrict__ ox,
+// each: per plane, 2 kPad full lines along the fast axis and n segments of
+// 2 kPad cells, n the extent of the slow one.  c_fast: cells ordered [b][c],
+// else [c][b].
+__global__ void cone_border_kernel(int P, int nx, int ny, int nz, int copies, bool c_fast, float *__restrict__ ox,
                                    float *__restrict__ oy, float *__restrict__ oz) {
     constexpr int W = 2 * kPad;
     for (int a = 0; a < copies; ++a) {
         const int na = a == 0 ? nx : (a == 1 ? ny : nz);
         const int nb = a == 0 ? ny : nx, nc = a == 2 ? ny : nz;
-        const int nbp = nb + W, ncp = nc + W;
+        const int ns = c_fast ? nb : nc, nf = c_fast ? nc : nb, nsp = ns + W, nfp = nf + W;
         float *o = a == 0 ? ox : (a == 1 ? oy : oz);
-        const int per = W * ncp + nb * W;                 // border cells of one plane
+        const int per = W * nfp + ns * W;                 // border cells of one plane
         const int64_t n = (int64_t)na * per;
         for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
             const int i = (int)(k / per), r = (int)(k - (int64_t)i * per);
-            int b, c;
-            if (r < W * ncp) {
-                b = r / ncp;
-                c = r - b * ncp;
-                if (b >= kPad) b += nb;
+            int s, f;
+            if (r < W * nfp) {
+                s = r / nfp;
+                f = r - s * nfp;
+                if (s >= kPad) s += ns;
             } else {
-                const int q = r - W * ncp;
-                b = kPad + q / W;
-                c = q % W;
-                if (c >= kPad) c += nc;
+                const int q = r - W * nfp;
+                s = kPad + q / W;
+                f = q % W;
+                if (f >= kPad) f += nf;
             }
-            float *d = o + (((int64_t)i * nbp + b) * ncp + c) * P;
+            float *d = o + (((int64_t)i * nsp + s) * nfp + f) * P;
             for (int m = 0; m < P; ++m) d[m] = 0.f;
         }
     }
@@ -87,14 +89,23 @@ __global__ void __launch_bounds__(kThreads)
     }
 }
 
-// Interior of the z-driven copy [iz][ix][iy] (plans with z-driven rays only).
-__global__ void cone_pack_z_kernel(const float *__restrict__ x, int nm, int P, int nx, int ny, int nz,
-                                   float *__restrict__ oz) {
+// Interiors of the copies ordered [c][b] (x fastest in the volume and in all but
+// the x-driven copy); oz only with z-driven rays.
+__global__ void cone_pack_rows_kernel(const float *__restrict__ x, int nm, int P, int nx, int ny, int nz,
+                                      float *__restrict__ ox, float *__restrict__ oy, float *__restrict__ oz) {
+    constexpr int W = 2 * kPad;
     const int64_t n = (int64_t)nx * ny * nz;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
         const int ix = (int)(j % nx), iy = (int)((j / nx) % ny), iz = (int)(j / ((int64_t)nx * ny));
-        float *d = oz + (((int64_t)iz * (nx + 2 * kPad) + ix + kPad) * (ny + 2 * kPad) + iy + kPad) * P;
-        for (int m = 0; m < P; ++m) d[m] = m < nm ? x[m * n + j] : 0.f;
+        float *dx = ox + (((int64_t)ix * (nz + W) + iz + kPad) * (ny + W) + iy + kPad) * P;
+        float *dy = oy + (((int64_t)iy * (nz + W) + iz + kPad) * (nx + W) + ix + kPad) * P;
+        float *dz = oz ? oz + (((int64_t)iz * (ny + W) + iy + kPad) * (nx + W) + ix + kPad) * P : nullptr;
+        for (int m = 0; m < P; ++m) {
+            const float v = m < nm ? x[m * n + j] : 0.f;
+            dx[m] = v;
+            dy[m] = v;
+            if (dz) dz[m] = v;
+        }
     }
 }
 
@@ -628,10 +639,23 @@ __global__ void __launch_bounds__(kThreads)
 
 }  // namespace
 
-mbir_status cone_pack(mbir_plan *p, const float *x, int nm, int P, bool z_too, cudaStream_t s) {
+mbir_status cone_pack_rows(mbir_plan *p, const float *x, int nm, int P, bool z_too, cudaStream_t s) {
     const mbir_geometry &g = p->g;
-    float *ox = p->xcol.p, *oy = p->xrow.p, *oz = p->xcol3.p;
-    cone_border_kernel<<<608, kThreads, 0, s>>>(P, g.nx, g.ny, g.nz, z_too ? 3 : 2, ox, oy, oz);
+    float *ox = p->xcol.p, *oy = p->xrow.p, *oz = z_too ? p->xcol3.p : nullptr;
+    cone_border_kernel<<<608, kThreads, 0, s>>>(P, g.nx, g.ny, g.nz, z_too ? 3 : 2, false, ox, oy, oz);
+    PSPS_LAUNCH_CHECK();
+    const int64_t b = cdiv(p->n_pix, kThreads);
+    cone_pack_rows_kernel<<<(unsigned)std::min<int64_t>(b, 65535 * 8), kThreads, 0, s>>>(x, nm, P, g.nx, g.ny, g.nz, ox, oy,
+                                                                                          oz);
+    PSPS_LAUNCH_CHECK();
+    return MBIR_OK;
+}
+
+// The copies ordered [b][c] that the columns read.
+static mbir_status cone_pack(mbir_plan *p, const float *x, int nm, int P, cudaStream_t s) {
+    const mbir_geometry &g = p->g;
+    float *ox = p->xcol.p, *oy = p->xrow.p;
+    cone_border_kernel<<<608, kThreads, 0, s>>>(P, g.nx, g.ny, g.nz, 2, true, ox, oy, nullptr);
     PSPS_LAUNCH_CHECK();
     const dim3 grd((unsigned)cdiv(g.nx, 32), (unsigned)g.ny, (unsigned)cdiv(g.nz, 32));
     if (P == 1)
@@ -641,10 +665,6 @@ mbir_status cone_pack(mbir_plan *p, const float *x, int nm, int P, bool z_too, c
     else
         cone_pack_kernel<4><<<grd, kThreads, 0, s>>>(x, nm, g.nx, g.ny, g.nz, (float4 *)ox, (float4 *)oy);
     PSPS_LAUNCH_CHECK();
-    if (z_too) {
-        cone_pack_z_kernel<<<2048, kThreads, 0, s>>>(x, nm, P, g.nx, g.ny, g.nz, oz);
-        PSPS_LAUNCH_CHECK();
-    }
     return MBIR_OK;
 }
 
@@ -670,6 +690,16 @@ mbir_status cone_cols_setup(mbir_plan *p) {
     const double drift = (0.5 * g.nz + 1.0) * std::sqrt(2.0) * std::max(g.dx, g.dy) / D * 0.5 * (kP - 1);
     const double need = 2.0 * (1.0 + drift) / k + 0.02;
     if (g.n_v >= (1 << 20)) return MBIR_OK;   // the row search's FP32 indices
+    // Its lanes run along z and every 32 layers cost the same, the tile scatter
+    // costs in proportion to the rows, above a floor per view that small
+    // images do not reach.  Two channels, us by tile / columns, as many rows as
+    // layers: 512 x 512 from 180 views 8 rows 2910 / 2850, 12 rows 3890 / 2860;
+    // 256 x 256 from 360 views 4 rows 1360 / 1850, 8 rows 1980 / 2020, 12 rows
+    // 2660 / 2030; 128 x 128 from 180 views 4 rows 325 / 284, 8 rows 428 / 282;
+    // four channels 256 x 256 8 rows 2450 / 2940, 12 rows 3350 / 2980, 128 x 128
+    // 4 rows 362 / 393, 8 rows 501 / 401; 64 x 64 from 90 views 4 rows 186 / 82.
+    const int64_t h = std::min<int64_t>(g.n_v / cdiv(g.nz, 32), g.nz);
+    if (h < 4 || (h < 12 && (int64_t)g.nx * g.ny * 12 > (h + 4) * 128 * 128)) return MBIR_OK;
     if (need > 48.0) return MBIR_OK;
     p->col_rows = need <= 4.0 ? std::max(2, (int)std::ceil(need)) : 6 * (int)std::ceil(need / 6.0);
     // View splits: enough warps for about three waves of 16 per SM, at least
@@ -683,10 +713,22 @@ mbir_status cone_cols_setup(mbir_plan *p) {
     return p->col_splits > 1 ? p->col_part.alloc((size_t)p->col_splits * 4 * p->n_pix) : MBIR_OK;
 }
 
+// A warp per detector column costs the same whatever the number of its rows
+// that meet the volume, a thread per ray in proportion to it.  256 x 256 voxels
+// from 360 x 512 columns, us per ray / columns, for as many rows (32 and 64
+// per warp) as layers: one material 24 rows 1500 / 1940, 32 rows 1970 / 1940,
+// 64 rows 3850 / 1950; two 12 rows 1090 / 1450, 16 rows 1440 / 1450, 24 rows
+// 2130 / 1460; four 16 rows 1910 / 1940, 24 rows 2840 / 1950.  The lines lie at
+// the same row counts for 64 to 512 voxels across and 60 to 360 views.
+bool cone_cols_forward(const mbir_geometry &g, int P) {
+    const double hit = std::min((double)g.n_v, g.nz * g.dz * g.sdd / (g.sid * g.dv));   // rows that meet the volume
+    return hit >= (P == 1 ? 32.0 : 17.0);
+}
+
 mbir_status project_cone_cols(mbir_plan *p, const float *x, float *l, int nm, cudaStream_t s) {
     const mbir_geometry &g = p->g;
     const int P = nm == 1 ? 1 : (nm == 2 ? 2 : 4);
-    PSPS_TRY(cone_pack(p, x, nm, P, false, s));
+    PSPS_TRY(cone_pack(p, x, nm, P, s));
     const int ncg = (int)cdiv(g.n_u, kFCols);
     auto run = [&](auto m, auto r) {
         constexpr int M = decltype(m)::value, R = decltype(r)::value;
@@ -703,12 +745,23 @@ mbir_status project_cone_cols(mbir_plan *p, const float *x, float *l, int nm, cu
         else
             run(m, r1);
     };
-    if (P == 1)
-        pick(std::integral_constant<int, 1>{}, std::integral_constant<int, 6>{}, std::integral_constant<int, 4>{});
-    else if (P == 2)
-        pick(std::integral_constant<int, 2>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, 3>{});
-    else
-        pick(std::integral_constant<int, 4>{}, std::integral_constant<int, 2>{}, std::integral_constant<int, 1>{});
+    // few rows: one chunk of 32 or 64, whose warps hold fewer idle rows
+    using std::integral_constant;
+    if (P == 1) {
+        if (g.n_v <= 64)
+            run(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+        else
+            pick(integral_constant<int, 1>{}, integral_constant<int, 6>{}, integral_constant<int, 4>{});
+    } else if (P == 2) {
+        if (g.n_v <= 32)
+            run(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+        else if (g.n_v <= 64)
+            run(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+        else
+            pick(integral_constant<int, 2>{}, integral_constant<int, 4>{}, integral_constant<int, 3>{});
+    } else {
+        pick(integral_constant<int, 4>{}, integral_constant<int, 2>{}, integral_constant<int, 1>{});
+    }
     PSPS_LAUNCH_CHECK();
     return MBIR_OK;
 }

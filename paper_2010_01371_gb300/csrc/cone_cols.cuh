@@ -34,8 +34,9 @@ __device__ __forceinline__ float cone_weight(const mbir_geometry &g, float2 W, f
 }
 
 // Packed copies of x[m][z][y][x] for each driving axis a, materials innermost
-// with stride P (1, 2 or 4): [a][b][c][m], c = z fastest (a = z: [iz][ix][iy]),
-// each plane with kPad zero cells on both sides of b and c.
+// with stride P (1, 2 or 4), each plane with kPad zero cells on both sides of
+// b and c.  The columns' lanes run along z and read [a][b][c], c = z fastest;
+// the general kernel's lanes run along the detector row and read [a][c][b].
 constexpr int kPad = 2;
 
 template <int NM>
@@ -56,9 +57,11 @@ struct CPack<4> {
     __device__ static void get(const T &v, float (&o)[4]) { o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w; }
 };
 
-// Volume copies of nm materials (P floats per cell) into the plan's scratch;
-// the copy of the z-driven rays only when z_too.
-mbir_status cone_pack(mbir_plan *p, const float *x, int nm, int P, bool z_too, cudaStream_t s);
+// Volume copies [a][c][b] of nm materials (P floats per cell) into the plan's
+// scratch; the copy of the z-driven rays only when z_too.
+mbir_status cone_pack_rows(mbir_plan *p, const float *x, int nm, int P, bool z_too, cudaStream_t s);
+// Whether the column forward pays for P materials (p->cols given).
+bool cone_cols_forward(const mbir_geometry &g, int P);
 // The column kernels' rules and buffers, decided once per plan.
 mbir_status cone_cols_setup(mbir_plan *p);
 // l[m] = A x[m] for nm <= 4 materials; x[c] (+)= A^T sino[c] for nc <= 4
