@@ -62,10 +62,15 @@ template void ls_fused_nm<PSPS_MODEL_NM>(SpecDev, int64_t, const float *, const 
 #else
 
 // More dynamic shared memory than a kernel gets without asking (the largest
-// spectra with eight channels).
-template <class K>
-static void allow_smem(K kernel, size_t bytes) {
-    if (bytes > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+// spectra with eight channels).  The limit belongs to the kernel, which every
+// plan and thread shares, so it is always the kernel's largest need, never the
+// call's: a call with a smaller spectrum must not lower it between another
+// thread's setting and its launch.  An error is left to the launch check.
+template <int NM, int CM, class K>
+static void allow_smem(K kernel) {
+    constexpr size_t most = sizeof(f32x2) * SpecTab<NM, CM>::Stride * kMaxE + sizeof(float) * ((CM + 3) & ~3) +
+                            sizeof(float) * 3 * CM * 2 * kModelThreads;
+    if constexpr (most > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 // Shared memory of the row kernels: the spectrum plus staging of two rays per
@@ -75,8 +80,8 @@ static void model_rows_cm(SpecDev sp, int64_t n, const float *l, const float *y,
                           float *kappa, dfloat *partials, int nblocks, cudaStream_t s) {
     const size_t sm = SpecTab<NM, CM>::bytes(sp.ne, sp.nc) +
                       sizeof(float) * (sp.noise.a > 0.f ? 3 : 2) * CM * 2 * kModelThreads;
-    allow_smem(model_grad_rows_kernel<NM, CM, true>, sm);
-    allow_smem(model_grad_rows_kernel<NM, CM, false>, sm);
+    allow_smem<NM, CM>(model_grad_rows_kernel<NM, CM, true>);
+    allow_smem<NM, CM>(model_grad_rows_kernel<NM, CM, false>);
     if (kappa)
         model_grad_rows_kernel<NM, CM, true><<<nblocks, kModelThreads, sm, s>>>(sp, n, l, y, gamma, g, kappa, partials);
     else
@@ -98,8 +103,8 @@ template <int NM, int CM>
 static void ls_rows_cm(SpecDev sp, int64_t n, const float *l, const float *q, const float *y, DevLS *ls, LsCfg cfg,
                        int mode, int last, dfloat *partials, int nblocks, cudaStream_t s) {
     const size_t sm = SpecTab<NM, CM>::bytes(sp.ne, sp.nc) + sizeof(float) * (mode == 0 ? 3 : 1) * CM * 2 * kModelThreads;
-    allow_smem(ls_rows_kernel<NM, CM, 0>, sm);
-    allow_smem(ls_rows_kernel<NM, CM, 1>, sm);
+    allow_smem<NM, CM>(ls_rows_kernel<NM, CM, 0>);
+    allow_smem<NM, CM>(ls_rows_kernel<NM, CM, 1>);
     if (mode == 0)
         ls_rows_kernel<NM, CM, 0><<<nblocks, kModelThreads, sm, s>>>(sp, n, l, q, y, ls, cfg, last, partials);
     else
