@@ -1233,10 +1233,16 @@ mbir_status project_2d_nm(mbir_plan *p, const float *x, float *l, cudaStream_t s
 
 }  // namespace
 
-// Angle between the outer rays of a warp of the strip forward (their
-// positions are then monotone in the bin); wider ones go ray by ray.
-static double strip_bins_span(const mbir_plan *p) {
-    return p->g.kind == MBIR_PAR2D ? 0.0 : 32.0 * p->g.du / p->g.sdd;
+// Whether the strip forward serves a scan; the others go ray by ray.  Its
+// staged samples are read without a bounds test, on the ground that a warp's
+// first and last ray bound the rows of those in between: the rays of one
+// driving axis span less than a right angle, so their positions are monotone
+// in the bin, and FP32 positions are within a row of the true ones.  They err
+// by a few 2^-24 of |f0| <= n (1 + aspect of the pixels): 0.1 rows at 16384
+// pixels and an aspect of 8, 127 rows at 1e5.
+static bool strips_serve(const mbir_geometry &g) {
+    const double span = g.kind == MBIR_PAR2D ? 0.0 : 32.0 * g.du / g.sdd;
+    return span < 1.5 && std::max(g.dx, g.dy) <= 8.0 * std::min(g.dx, g.dy);
 }
 
 mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStream_t s) {
@@ -1265,7 +1271,7 @@ mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStrea
         const int nm = n_mat - m0 < 4 ? n_mat - m0 : 4;
         const float *xm = x + (int64_t)m0 * p->n_pix;
         float *lm = l + (int64_t)m0 * p->n_rays;
-        if (p->fwd_mode == 2 && strip_bins_span(p) < 1.5) {
+        if (p->fwd_mode == 2 && strips_serve(p->g)) {
             switch (nm) {
                 case 1: PSPS_TRY(project_strip_nm<1>(p, xm, lm, s)); break;
                 case 2: PSPS_TRY(project_strip_nm<2>(p, xm, lm, s)); break;
@@ -1421,14 +1427,16 @@ extern "C" mbir_status mbir_plan_create(const mbir_geometry *g, int n_mat_max, m
         // three 474 / 389; 320^2 from 720 x 556 86 / 86 and 235 / 188; 256^2 from
         // 360 x 444 (630 CTAs) 41 / 58 and 93 / 99.  On a driving plane adjacent
         // rays are at most sqrt2 du (1 + R / sid) sid / sdd / pixel apart (fan;
-        // du for parallel beam), a ray moves at most one row per driving index,
-        // and the CTA's views turn by their spacing each.
+        // du for parallel beam), a ray moves at most the pixels' aspect in rows per
+        // driving index, and the CTA's views turn by their spacing each.
         const mbir_geometry &q = p->g;
         const double pix = std::min(q.dx, q.dy), R = std::hypot(0.5 * q.nx * q.dx, 0.5 * q.ny * q.dy);
         const double d = std::sqrt(2.0) * (q.kind == MBIR_PAR2D ? q.du : q.du * (q.sid + R) / q.sdd) / pix;
         const double turn = std::sqrt(2.0) * R / pix * std::fabs(q.angle_span) / q.n_views;
         const int64_t ctas = cdiv(q.n_u, 32) * cdiv(q.n_views, kThreads / 32);
-        if (ctas >= 152 * 8 && 32 * d + (kThreads / 32 - 1) * turn + 32.0 + 8.0 <= kSH) p->fwd_mode = 2, p->strip_bins = 32;
+        const double aspect = std::max(q.dx, q.dy) / pix;
+        if (strips_serve(q) && ctas >= 152 * 8 && 32 * d + (kThreads / 32 - 1) * turn + 32.0 * aspect + 8.0 <= kSH)
+            p->fwd_mode = 2, p->strip_bins = 32;
     }
     {
         // default views per CTA of the tile transpose: about six CTAs per SM
