@@ -173,7 +173,12 @@ mbir_status mbir_plan_set_strip_bins(mbir_plan *plan, int bins);
 mbir_status mbir_plan_set_cone_tile(mbir_plan *plan, int depth);
 /* The plan's current choices (any pointer may be NULL): forward algorithm
  * (mbir_plan_set_projector's modes), strip bins per CTA, transpose mode,
- * tile-transpose views per CTA (2-D) and cone tile depth (3-D). */
+ * tile-transpose views per CTA (2-D) and cone tile depth (3-D).  A choice that
+ * the plan has no use for is reported as it was set: the forward algorithm and
+ * the tile depth of a cone plan that runs over detector columns; and forward 2
+ * is the default of 2-D scans with many rays, where small images (below 192^2
+ * pixels, 352^2 for one or four images at a time) go ray by ray all the same
+ * until mbir_plan_set_projector or mbir_plan_autotune chooses. */
 mbir_status mbir_plan_tuning(const mbir_plan *plan, int *fwd_mode, int *strip_bins, int *back_mode, int *back_views,
                              int *cone_tile);
 /* Select the forward projector's algorithm (Eq. 1's A).  2-D: 0 = per-tile

@@ -228,7 +228,8 @@ struct mbir_plan {
     psps::DBuf<float4> view;      // parallel: (cos, sin, -, -); fan: (sx, sy, beta + pi, -)
     int back_mode = 0;            // 0 default (2-D tile scatter; 3-D columns or tile scatter), 1 pixel / voxel gather, 2 ray-driven atomics, 3 split-table gather (3-D)
     int back_views = 60;          // views per CTA of the tile transpose
-    int fwd_mode = 1;             // 0 tile sums, 1 one thread per ray (default), 2 shared-memory strips
+    int fwd_mode = 1;             // 0 tile sums, 1 one thread per ray, 2 shared-memory strips (default of large scans)
+    bool fwd_default = true;      // nobody chose it: strips only for images where they pay
     int strip_bins = 64;          // strip forward: bins per CTA (32, 64, 128 or 256; 256 / it views)
     // 3-D per-ray Joseph set-up (cone_ray, computed once; general kernels): (fb_mid, dfb,
     // fc_mid, dfc) in `ray` and (weight, bits(axis | lo << 2 | hi << 17)) in

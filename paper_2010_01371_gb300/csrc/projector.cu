@@ -1245,6 +1245,19 @@ static bool strips_serve(const mbir_geometry &g) {
     return span < 1.5 && std::max(g.dx, g.dy) <= 8.0 * std::min(g.dx, g.dy);
 }
 
+// Whether strips, left as the plan's default, pay for nm images: small images
+// have few strips per ray to spread a CTA's set-up over, and with one or four
+// images the per-ray kernels are the better ones for longer.  720 or 1440 views,
+// 1.4 to 3 bins per pixel, time per ray / strips for 1, 2, 3 and 4 images: fan beam
+// 128^2 0.72-0.83, 0.82-0.92, 0.95-1.12, 0.86-0.91; 192^2 0.91-0.93, 1.02-1.18,
+// 1.10-1.15, 0.94-0.99; 256^2 0.93-0.96, 1.08-1.16, 1.13-1.21, 0.94-1.01; 320^2
+// 0.98-1.03, 1.09-1.16, 1.12-1.24, 0.97-0.99; 384^2 1.01-1.05, 1.18-1.25,
+// 1.16-1.24, 0.98-1.03; parallel beam a few per cent more.
+static bool strips_pay(const mbir_geometry &g, int nm) {
+    const int64_t side = nm == 1 || nm == 4 ? 352 : 192;
+    return (int64_t)g.nx * g.ny >= side * side;
+}
+
 mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStream_t s) {
     if (p->g.kind == MBIR_CONE3D) return project_cone(p, x, l, n_mat, s);
     if (p->fwd_mode == 0) {
@@ -1271,7 +1284,7 @@ mbir_status project(mbir_plan *p, const float *x, float *l, int n_mat, cudaStrea
         const int nm = n_mat - m0 < 4 ? n_mat - m0 : 4;
         const float *xm = x + (int64_t)m0 * p->n_pix;
         float *lm = l + (int64_t)m0 * p->n_rays;
-        if (p->fwd_mode == 2 && strips_serve(p->g)) {
+        if (p->fwd_mode == 2 && strips_serve(p->g) && (!p->fwd_default || strips_pay(p->g, nm))) {
             switch (nm) {
                 case 1: PSPS_TRY(project_strip_nm<1>(p, xm, lm, s)); break;
                 case 2: PSPS_TRY(project_strip_nm<2>(p, xm, lm, s)); break;
@@ -1571,6 +1584,7 @@ mbir_status autotune_impl(mbir_plan *p, int n_channels, cudaStream_t s) {
     // 2-D forward: one thread per ray, or the strip kernel with 32 .. 256
     // bins per CTA
     best_ms = 3.0e38f;
+    p->fwd_default = false;
     int best_mode = p->fwd_mode, best_sb = p->strip_bins;
     for (int c = 0; c < 5; ++c) {
         p->fwd_mode = c == 0 ? 1 : 2;
@@ -1594,10 +1608,11 @@ extern "C" mbir_status mbir_plan_autotune(mbir_plan *p, int n_channels, mbir_str
     if (cap != cudaStreamCaptureStatusNone) return fail(MBIR_ERR_ARG, "mbir_plan_autotune: stream is capturing");
     const int back_mode = p->back_mode, back_views = p->back_views, fwd_mode = p->fwd_mode, sb = p->strip_bins;
     const int cone_tile = p->cone_tile;
+    const bool fwd_default = p->fwd_default;
     const mbir_status st = autotune_impl(p, n_channels, s);
     if (st != MBIR_OK) {   // keep the plan as it was
         p->back_mode = back_mode, p->back_views = back_views, p->fwd_mode = fwd_mode, p->strip_bins = sb;
-        p->cone_tile = cone_tile;
+        p->cone_tile = cone_tile, p->fwd_default = fwd_default;
         return st;
     }
     if (views_per_cta) *views_per_cta = p->back_views;
@@ -1632,5 +1647,6 @@ extern "C" mbir_status mbir_plan_tuning(const mbir_plan *p, int *fwd_mode, int *
 extern "C" mbir_status mbir_plan_set_projector(mbir_plan *p, int mode) {
     if (!p || mode < 0 || mode > 2) return fail(MBIR_ERR_ARG, "mbir_plan_set_projector: bad argument");
     p->fwd_mode = mode;
+    p->fwd_default = false;
     return MBIR_OK;
 }
