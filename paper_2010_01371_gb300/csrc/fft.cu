@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kThreads)
 // Z[b], inverse in y.  Against separate passes Z is read and written once
 // instead of three times and two launches go; with the divisions above, a
 // 448^2 apply of three materials went from 79 to 65 us (same bits).
-constexpr int kMixThreads = 512;
+constexpr int kMixThreads = 512, kMixSmem = 128 * 1024;
 
 __global__ void __launch_bounds__(kMixThreads)
     fft_mix_kernel(int N, int B, int nx, int nm, Radices rad, float2 *__restrict__ Z, const float *__restrict__ L,
@@ -392,14 +392,23 @@ mbir_status FftPlan::inverse(int channels, float2 *Z, float *out, const float *p
 
 mbir_status FftPlan::mixed(int channels, const float *in, float2 *Z, float *out, const float *L, bool &done,
                            cudaStream_t s) const {
-    // four columns (whole sectors) per CTA where that gives every SM one,
-    // else two; more shared memory than a CTA has: the separate passes
-    const int B = nx >= 4 * 152 ? 4 : 2;
-    const size_t smem = 2 * sizeof(float2) * (size_t)ny * B * channels;
-    done = nz <= 1 && channels <= 4 && smem <= 200 * 1024 && (int64_t)ny * B * channels < 65536;
+    // Four columns (whole sectors) per CTA where that gives every SM one CTA
+    // and leaves room for two, else two.  A CTA whose columns take most of an
+    // SM's shared memory hides no latency; with many columns the separate
+    // passes are then faster.  us, separate / two / four columns: 630^2, two
+    // materials 96 / 96 / 92, three 133 / 137 / 159, four 133 / 147 / 170; 700^2, four
+    // 141 / 163 / 184; 768^2, two 122 / 111 / 110, three 180 / 170 / 207; 1024^2, two 201 /
+    // 182 / 197, four 336 / 382 / -; with fewer columns, 600^2, three 111 / 100 / 108;
+    // 256 x 1024, four 110 / 106 / -.
+    auto bytes = [&](int B) { return 2 * sizeof(float2) * (size_t)ny * B * channels; };
+    const bool wide = nx >= 4 * 152;
+    const int B = wide && bytes(4) <= 96 * 1024 ? 4 : 2;
+    const size_t smem = bytes(B);
+    done = nz <= 1 && channels <= 4 && (B == 4 || smem <= (wide ? 64 : kMixSmem / 1024) * 1024) &&
+           (int64_t)ny * B * channels < 65536;
     if (!done) return MBIR_OK;
     PSPS_TRY(run(0, 0, channels, in, Z, nullptr, nullptr, nullptr, s));
-    PSPS_CUDA(cudaFuncSetAttribute(fft_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    PSPS_CUDA(cudaFuncSetAttribute(fft_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem));
     Radices rad;
     factor(ny, rad);
     fft_mix_kernel<<<(unsigned)cdiv(nx, B), kMixThreads, smem, s>>>(ny, B, nx, channels, rad, Z, L, twy.p);
