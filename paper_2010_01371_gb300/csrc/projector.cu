@@ -941,12 +941,13 @@ __global__ void __launch_bounds__(kThreads, 8)
 // Weights and the sample split are the per-ray table's, as in every other
 // projector and transpose, so the result is the same operator.
 // Bound by issue (67-78 %) and shared-memory wavefronts (two or three per
-// sample and material).  512^2 from 720 x 888 rays, three images: 474 -> 389 us
-// against 16-byte gathers per ray, one image 171 -> 162; 448^2 from 720 x 780,
-// three images 387 -> 313.
+// sample and material).  512^2 from 720 x 888 rays, one image: 171 -> 162 us
+// against gathers per ray; 448^2 from 720 x 780, three images 387 -> 316.
+// Sixteen samples per compensated add are 0.7 % faster, and up to 0.6 % further
+// from the 64-bit projection than the gathers (eight: 0.3 %).
 constexpr int kSH = 160;           // staged window rows
 constexpr int kStripGroup = 16;    // strips whose windows are found together
-constexpr int kSub = 16;           // samples per compensated add
+constexpr int kSub = 8;            // samples per compensated add
 
 template <int NM>
 struct StripShape {
