@@ -32,7 +32,7 @@ def sources():
 
 
 # model_inst.cu instantiates the model kernels of one material count and one
-# family per compilation (96 kernel variants in all), so it is compiled once
+# family per compilation (128 kernel variants in all), so it is compiled once
 # per (count, family) pair and the pairs build in parallel.
 MODEL_INST = "model_inst.cu"
 

@@ -2,7 +2,7 @@
 // with SPS numerators and the fused line-search evaluation, plain and with
 // rays coupled along detector rows.  Each material count is instantiated in
 // its own translation unit (model_inst.cu compiled once per count and
-// family), so the 96 kernel variants compile in parallel.
+// family), so the 128 kernel variants compile in parallel.
 #pragma once
 #include <cmath>
 
@@ -30,9 +30,12 @@ __device__ __forceinline__ float transmission(float z) { return exp2f(z * -1.442
 // The energy loops take two rays per thread, as the two halves of packed FP32
 // pairs, which halves the issue slots of everything but the exponentials.
 // Their table holds, per energy, every factor twice (one 16-byte shared-memory
-// load brings two of them, for both rays): q_m = -log2(e) Q[E][m] (the sum
-// over m is then the exponent of 2; factors of log2 e leave per ray), then
-// S[c][E].
+// load brings two of them, for both rays): Q[E][m], then S[c][E].  The exponent
+// -log2(e) z of 2 is one more product per energy.  Putting the factor into the
+// table (error of a one-energy gradient 7.8e-8 instead of 4.0e-8) or into the
+// line integrals (two materials: 3.30e-7 instead of 3.17e-7, since a rounded
+// line integral errs alike at every energy) saves that, 3 % of a
+// projection-domain iteration.
 // Measured on 720 x 888 rays, 2 materials, 121 energies, 2 channels (ncu, cold):
 // numerators 117 -> 80 us, line-search evaluation 76 -> 55 us, the eight halving
 // candidates 181 -> 107 us against one ray per thread with exp2f's subnormal
@@ -41,9 +44,10 @@ __device__ __forceinline__ float transmission(float z) { return exp2f(z * -1.442
 // correlated noise the data-term gradient 174 -> 96 us.  The FP32 pipe is half
 // busy and so is issue (50 % each for the evaluation); more rays (x 8) run at
 // the same rate.
-constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kLog2eHi = (float)1.4426950408889634;                            // log2(e) = hi + lo
-constexpr float kLog2eLo = (float)(1.4426950408889634 - (double)(float)1.4426950408889634);
+constexpr float kLog2e = 1.4426950408889634f;
+
+// Exponents of 2 that give exp(-z).
+__device__ __forceinline__ f32x2 neglog2e(f32x2 z) { return mul2(z, pair2(-kLog2e, -kLog2e)); }
 
 template <int NM, int CM>
 struct SpecTab {
@@ -64,8 +68,7 @@ struct SpecTab {
             const int e = i / Stride, k = i - e * Stride;
             float v = 0.f;
             if (k < NM) {
-                const float Q = sp.qs[e * NM + k];
-                v = fmaf(-kLog2eHi, Q, -kLog2eLo * Q);
+                v = sp.qs[e * NM + k];
             } else if (k - NM < nc) {
                 v = S[(k - NM) * ne + e];
             }
@@ -170,7 +173,7 @@ __device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s;
                 tab.get(e, c, q, s);
-                a = fma2(s, exp2_pair(dot2(q, l)), a);
+                a = fma2(s, exp2_pair(neglog2e(dot2(q, l))), a);
             }
             put(yb, c, a);
         },
@@ -179,7 +182,7 @@ __device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s[CM];
                 tab.get(e, q, s);
-                const f32x2 t = exp2_pair(dot2(q, l));
+                const f32x2 t = exp2_pair(neglog2e(dot2(q, l)));
 #pragma unroll
                 for (int c = 0; c < CM; ++c) yb[c] = fma2(s[c], t, yb[c]);
             }
@@ -197,9 +200,9 @@ __device__ __forceinline__ void numerators2(const SpecTab<NM, CM> &tab, const f3
 #pragma unroll
     for (int m = 0; m < NM; ++m) gm[m] = km[m] = 0ull;
     auto add = [&](const f32x2 (&q)[NM], f32x2 nv, f32x2 eta) {
-        const f32x2 t = exp2_pair(dot2(q, l)), tv = mul2(t, nv);
+        const f32x2 t = exp2_pair(neglog2e(dot2(q, l))), tv = mul2(t, nv);
 #pragma unroll
-        for (int m = 0; m < NM; ++m) gm[m] = fma2(q[m], tv, gm[m]);   // (-log2(e) Q) (-t v)
+        for (int m = 0; m < NM; ++m) gm[m] = fma2(q[m], tv, gm[m]);   // Q (-t v)
         if constexpr (KAPPA) {
             const f32x2 nrho = fma2(eta, t, nv), uh = max2(t, 1.f);
             const f32x2 cE = max2(mul2(sub2(mul2(add2(eta, eta), uh), nrho), uh), 0.f);
@@ -228,24 +231,18 @@ __device__ __forceinline__ void numerators2(const SpecTab<NM, CM> &tab, const f3
             }
         },
         [](int, int) {});
-    const f32x2 c1 = pair2(-kLn2, -kLn2), c2 = pair2(kLn2 * kLn2, kLn2 * kLn2);
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-        gm[m] = mul2(gm[m], c1);
-        if constexpr (KAPPA) km[m] = mul2(km[m], c2);
-    }
 }
 
-// Counts at l and their first two derivatives along q (in units of alpha), and
-// the largest exponent of 2 met (-log2(e) times the smallest z), all energies.
+// Counts at l and their first two derivatives along -ndir, and the
+// largest exponent of 2 met (-log2(e) times the smallest z), all energies.
 template <int NM, int CM>
-__device__ __forceinline__ void line2(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], const f32x2 (&dir)[NM],
+__device__ __forceinline__ void line2(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], const f32x2 (&ndir)[NM],
                                       f32x2 (&yb)[CM], f32x2 (&d1)[CM], f32x2 (&d2)[CM], float &za, float &zb) {
 #pragma unroll
     for (int c = 0; c < CM; ++c) yb[c] = d1[c] = d2[c] = 0ull;
     za = zb = -3.0e38f;
     auto exponent = [&](const f32x2 (&q)[NM]) {
-        const f32x2 z = dot2(q, l);
+        const f32x2 z = neglog2e(dot2(q, l));
         float a, b;
         unpair2(z, a, b);
         za = fmaxf(za, a), zb = fmaxf(zb, b);
@@ -259,7 +256,7 @@ __device__ __forceinline__ void line2(const SpecTab<NM, CM> &tab, const f32x2 (&
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s;
                 tab.get(e, c, q, s);
-                const f32x2 t = exp2_pair(exponent(q)), dz = dot2(q, dir), tdz = mul2(t, dz);
+                const f32x2 t = exp2_pair(exponent(q)), dz = dot2(q, ndir), tdz = mul2(t, dz);
                 a = fma2(s, t, a);
                 b = fma2(s, tdz, b);
                 d = fma2(s, mul2(tdz, dz), d);
@@ -271,7 +268,7 @@ __device__ __forceinline__ void line2(const SpecTab<NM, CM> &tab, const f32x2 (&
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s[CM];
                 tab.get(e, q, s);
-                const f32x2 t = exp2_pair(exponent(q)), dz = dot2(q, dir), tdz = mul2(t, dz), td2 = mul2(tdz, dz);
+                const f32x2 t = exp2_pair(exponent(q)), dz = dot2(q, ndir), tdz = mul2(t, dz), td2 = mul2(tdz, dz);
 #pragma unroll
                 for (int c = 0; c < CM; ++c) {
                     yb[c] = fma2(s[c], t, yb[c]);
@@ -287,10 +284,6 @@ __device__ __forceinline__ void line2(const SpecTab<NM, CM> &tab, const f32x2 (&
                 exponent(q);
             }
         });
-    // dz = -log2(e) dz/dalpha: d/dalpha of t is (ln 2) (dz) t
-    const f32x2 c1 = pair2(kLn2, kLn2), c2 = pair2(kLn2 * kLn2, kLn2 * kLn2);
-#pragma unroll
-    for (int c = 0; c < CM; ++c) d1[c] = mul2(d1[c], c1), d2[c] = mul2(d2[c], c2);
 }
 
 // Counts at l + alpha_k dir for K steps alpha_k at once (the exponents are
@@ -310,7 +303,7 @@ __device__ __forceinline__ void candidates2(const SpecTab<NM, CM> &tab, const f3
     for (int e = 0; e < tab.ne; ++e) {
         f32x2 q[NM], s[CM];
         tab.get(e, q, s);
-        const f32x2 z0 = dot2(q, l), z1 = dot2(q, dir);
+        const f32x2 z0 = neglog2e(dot2(q, l)), z1 = neglog2e(dot2(q, dir));
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const f32x2 z = fma2(al[k], z1, z0);
@@ -373,7 +366,7 @@ struct SegPair {
     }
 };
 
-// Largest exponent of 2 met over all energies (see line2).
+// Largest exponent of 2 met over all energies.
 template <int NM, int CM>
 __device__ __forceinline__ void top_exponent(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], float &za, float &zb) {
     za = zb = -3.0e38f;
@@ -381,7 +374,7 @@ __device__ __forceinline__ void top_exponent(const SpecTab<NM, CM> &tab, const f
         f32x2 q[NM], s;
         tab.get(e, 0, q, s);
         float a, b;
-        unpair2(dot2(q, l), a, b);
+        unpair2(neglog2e(dot2(q, l)), a, b);
         za = fmaxf(za, a), zb = fmaxf(zb, b);
     }
 }
@@ -471,7 +464,7 @@ __global__ void __launch_bounds__(kModelThreads)
     tab.load(sp, spec_smem4);
     const int nc = sp.nc;
     const int nh = cfg.n_halve < kMaxHalve ? cfg.n_halve : kMaxHalve;
-    const float z_lim = cfg.z_min * -kLog2eHi;   // exponents above it leave the domain
+    const float z_lim = cfg.z_min * -kLog2e;   // exponents above it leave the domain
     constexpr int NACC = MODE == 0 ? 4 : 2 * kMaxHalve;
     dfloat acc[NACC];
 #pragma unroll
@@ -479,11 +472,11 @@ __global__ void __launch_bounds__(kModelThreads)
     if constexpr (MODE == 0) {
         const f32x2 alpha2 = pair2(alpha, alpha);
         do {
-            f32x2 la[NM], yb[CM], d1[CM], d2[CM];
+            f32x2 la[NM], nq[NM], yb[CM], d1[CM], d2[CM];
             float za, zb;
 #pragma unroll
-            for (int m = 0; m < NM; ++m) la[m] = fma2(alpha2, qm[m], lm[m]);
-            line2(tab, la, qm, yb, d1, d2, za, zb);
+            for (int m = 0; m < NM; ++m) la[m] = fma2(alpha2, qm[m], lm[m]), nq[m] = sub2(0ull, qm[m]);
+            line2(tab, la, nq, yb, d1, d2, za, zb);
             float f[2] = {0.f, 0.f}, f1[2] = {0.f, 0.f}, f2[2] = {0.f, 0.f};
 #pragma unroll
             for (int c = 0; c < CM; ++c)
@@ -816,7 +809,7 @@ __global__ void __launch_bounds__(kModelThreads)
     SpecTab<NM, CM> tab;
     tab.load(sp, spec_smem4);
     const int nc = sp.nc;
-    const float z_lim = cfg.z_min * -kLog2eHi;
+    const float z_lim = cfg.z_min * -kLog2e;
     // [NV][CM][B] with NV = 3 values per channel and ray (mode 0) or 1
     float *buf = reinterpret_cast<float *>(reinterpret_cast<char *>(spec_smem4) + SpecTab<NM, CM>::bytes(sp.ne, nc));
     const int B = 2 * blockDim.x;
@@ -855,8 +848,12 @@ __global__ void __launch_bounds__(kModelThreads)
                 f32x2 la[NM], v0[CM], v1[CM], v2[CM];
 #pragma unroll
                 for (int m = 0; m < NM; ++m) la[m] = fma2(pair2(ak, ak), qm[m], lm[m]);
-                if constexpr (MODE == 0)
-                    line2(tab, la, qm, v0, v1, v2, ze[0], ze[1]);
+                if constexpr (MODE == 0) {
+                    f32x2 nq[NM];
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) nq[m] = sub2(0ull, qm[m]);
+                    line2(tab, la, nq, v0, v1, v2, ze[0], ze[1]);
+                }
                 else {
                     counts2(tab, la, v0);
                     top_exponent(tab, la, ze[0], ze[1]);
