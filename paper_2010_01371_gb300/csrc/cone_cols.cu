@@ -781,21 +781,21 @@ mbir_status backproject_cols(mbir_plan *p, const float *sino, float *x, int nc, 
     const dim3 grd((unsigned)(cdiv(g.nx, kBX * kP) * cdiv(g.ny, kBY * kP) * cdiv(g.nz, 32)), (unsigned)ns);
     float *dst = ns > 1 ? p->col_part.p : x;
     const int64_t stride = ns > 1 ? (int64_t)4 * p->n_pix : 0;
-    auto run = [&](auto nr, auto multi) {
+    auto run = [&](auto nr, auto multi) -> mbir_status {
         constexpr size_t smem = kBWarps * (sizeof(ColDesc) + (sizeof(f32x2) + sizeof(unsigned)) * (kP * kP * C / 2) * 32);
-        cudaFuncSetAttribute(back_cols_kernel<C, decltype(nr)::value, decltype(multi)::value>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        back_cols_kernel<C, decltype(nr)::value, decltype(multi)::value><<<grd, 32 * kBWarps, smem, s>>>(
-            g, p->view.p, p->view_cols.p, p->col.p, p->colw.p, p->wsino.p, p->wmax.p, p->col_rows, p->col_vchunk, nc,
-            dst, stride, accumulate);
+        constexpr auto kernel = back_cols_kernel<C, decltype(nr)::value, decltype(multi)::value>;
+        PSPS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kernel<<<grd, 32 * kBWarps, smem, s>>>(g, p->view.p, p->view_cols.p, p->col.p, p->colw.p, p->wsino.p, p->wmax.p,
+                                               p->col_rows, p->col_vchunk, nc, dst, stride, accumulate);
+        PSPS_LAUNCH_CHECK();
+        return MBIR_OK;
     };
     switch (p->col_rows) {
-        case 2: run(std::integral_constant<int, 2>{}, std::false_type{}); break;
-        case 3: run(std::integral_constant<int, 3>{}, std::false_type{}); break;
-        case 4: run(std::integral_constant<int, 4>{}, std::false_type{}); break;
-        default: run(std::integral_constant<int, 6>{}, std::true_type{}); break;   // passes of 6
+        case 2: PSPS_TRY(run(std::integral_constant<int, 2>{}, std::false_type{})); break;
+        case 3: PSPS_TRY(run(std::integral_constant<int, 3>{}, std::false_type{})); break;
+        case 4: PSPS_TRY(run(std::integral_constant<int, 4>{}, std::false_type{})); break;
+        default: PSPS_TRY(run(std::integral_constant<int, 6>{}, std::true_type{})); break;   // passes of 6
     }
-    PSPS_LAUNCH_CHECK();
     if (ns > 1) {
         const int64_t n = (int64_t)nc * p->n_pix, b = cdiv(n, kThreads);
         cols_reduce_kernel<<<(unsigned)(b < 4096 ? b : 4096), kThreads, 0, s>>>(p->col_part.p, ns, stride, n, x,
