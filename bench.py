@@ -306,6 +306,14 @@ def cpu_baseline(workload: str, kind: str, prob, n_iter: int, views=None, scale:
                       f"rate" + (f", scaled by {scale:.4g} to the full scan" if scale != 1.0 else "")}
 
 
+def plan_choices(plan):
+    """The tuning choices that act on a plan's calls (a cone plan over detector columns has one, its transpose)."""
+    if plan is None:
+        return None
+    t = plan.tuning()
+    return {"backproject_mode": t["backproject_mode"]} if plan.geom.kind == 2 else t
+
+
 def reference_arm(args):
     rank, world, _ = dist_env()
     if rank != 0:
@@ -488,7 +496,7 @@ def ours(args, prob, workload=WORKLOAD, kind="haar", desc="", blur=None, noise=N
             "config": {"workload": workload, "problem": desc or WORKLOADS[workload][2], "precond": kind,
                        "line_search": True, "graph": True,
                        "l2": "flushed (256 MB write) between timed steps", "build_s": round(build_s, 3),
-                       "views_per_cta": tuned, "tuning": plan.tuning() if plan is not None else None},
+                       "views_per_cta": tuned, "tuning": plan_choices(plan)},
             "gpu_launches": launches, "clocks": clk, "roofline": roofline,
             "e2e": {"value": world * args.steps / e2e_s, "unit": "iter/s",
                     "h2d_bytes_per_step": int(y_host.numel() * 4), "d2h_bytes_per_step": 2 * 8 + DEVLS_BYTES}}
@@ -684,7 +692,7 @@ def kernel_bench(args, prob):
     out = {}
     if prob.geom.kind == 2:
         # cone beam: forward of the basis images, and the 2 n_mat-channel
-        # transposes (fixed-point tile scatter, direct and split-table gathers)
+        # transposes (the plan's default, direct and split-table gathers)
         nm = x1.shape[0]
         s4 = torch.as_tensor(rng.random((2 * nm, plan.n_rays)).astype(np.float32), device=dev)
         l = torch.empty((nm, plan.n_rays), device=dev)
@@ -702,13 +710,10 @@ def kernel_bench(args, prob):
                 torch.cuda.synchronize()
                 ts.append(e0.elapsed_time(e1))
             return float(np.median(ts))
-        for mode in ["ray", "aligned"]:
-            plan.set_projector(mode)
-            out[f"project_{mode}_{nm}ch_ms"] = timec(lambda: p.mbir_project(plan, x1, l))
-        for mode in ["tile", "tile8", "gather", "split"]:
-            plan.set_backprojector("tile" if mode == "tile8" else mode)
-            plan.set_cone_tile(8 if mode == "tile8" else 16)
-            out[f"backproject_{mode}_{2 * nm}ch_ms"] = timec(lambda: p.mbir_backproject(plan, s4, img))
+        out[f"project_{nm}ch_ms"] = timec(lambda: p.mbir_project(plan, x1, l))
+        for mode, name in [("tile", "default"), ("gather", "gather"), ("split", "split")]:
+            plan.set_backprojector(mode)
+            out[f"backproject_{name}_{2 * nm}ch_ms"] = timec(lambda: p.mbir_backproject(plan, s4, img))
         print(json.dumps({"kernels": out, "workload": args.workload}), flush=True)
         return
     s2 = torch.as_tensor(rng.random((2, plan.n_rays)).astype(np.float32), device=dev)

@@ -99,7 +99,8 @@ int64_t mbir_plan_n_pix(const mbir_plan *plan);
 
 /* l[m] = A x[m] for m < n_mat (the operator A inside the exponential,
  * Sec. II-D; for one-step MBMD, A is applied per basis material, Sec. II-F).
- * x: [n_mat][image], l: [n_mat][n_rays] (overwritten). */
+ * x: [n_mat][image], l: [n_mat][n_rays] (overwritten).  A ray through a
+ * non-finite pixel or voxel comes out non-finite: NaN, or infinite. */
 mbir_status mbir_project(mbir_plan *plan, const float *x, float *l, int n_mat, mbir_stream stream);
 
 /* x[m] (+)= A^T s[m]: the exact transpose of mbir_project (same weights).
@@ -186,10 +187,13 @@ mbir_status mbir_plan_tuning(const mbir_plan *plan, int *fwd_mode, int *strip_bi
  * (tile, ray); 1 = one thread per ray with Kahan-compensated sums, gathering
  * from L1/L2, eight samples summed before each compensated add
  * (deterministic); 2 = rays of a block of views and bins march
- * shared-memory strips of the image, every lane on the same driving index
- * (deterministic).  Cone beam: one algorithm whatever the mode (a warp per
+ * shared-memory strips of the image, every lane on the same driving index,
+ * eight samples summed before each compensated add (deterministic; scans whose
+ * pixels are more than 8 times as long as wide, or whose 32 neighbouring bins
+ * span more than 1.5 rad, go ray by ray).  Cone beam: one algorithm whatever the mode (a warp per
  * detector column, lanes on its rows; one thread per ray for plans with rays
- * that the z axis drives or with few rows that meet the volume).  All use the same per-ray Joseph weights.
+ * that the z axis drives or with few rows that meet the volume).  All use the
+ * same per-ray Joseph weights.
  * MBIR_ERR_ARG for other modes. */
 mbir_status mbir_plan_set_projector(mbir_plan *plan, int mode);
 
@@ -245,7 +249,9 @@ mbir_status mbmd_forward_model(const mbmd_spectrum *spec, const float *l, float 
  * (Eq. 3, Sigma_y = diag(max(y,1))), y_bar as in mbmd_forward_model.  plan != NULL: x_or_l is an image
  * [n_mat][image] and l = A x is formed internally; plan == NULL: x_or_l is
  * the line-integral array [n_mat][n_rays] (projection-domain decomposition).
- * *objective is a DEVICE double written with the FP64-reduced value. */
+ * *objective is a DEVICE double written with the FP64-reduced value.  Here and
+ * in every derivative and line search a transmission exp(-Q l) below 2^-126
+ * counts as zero. */
 mbir_status mbmd_objective(mbir_plan *plan, const mbmd_spectrum *spec, const float *x_or_l, const float *y,
                            int64_t n_rays, double *objective, mbir_stream stream);
 
