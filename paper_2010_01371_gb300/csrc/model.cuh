@@ -78,7 +78,12 @@ constexpr int kModelMaxBlocks = 2048;  // partial sums per block at most
 inline int model_blocks(int64_t n) {
     const int64_t steps = cdiv(n, 2 * kModelThreads);
     static_assert(152 * 8 <= kModelMaxBlocks, "partials");
-    if (steps <= 152 * 8) return (int)(steps < 1 ? 1 : steps);
+    // small scans: a block for every segment of the row-coupled kernels too,
+    // whose halos take up to 14 of a step's rays (a block with two segments
+    // takes twice as long as all others: 20000 blurred rays, 6 channels 66 us for
+    // the gradient, 59 with a block each)
+    const int64_t segs = cdiv(n, 2 * kModelThreads - 14);
+    if (segs <= 152 * 8) return (int)(segs < 1 ? 1 : segs);
     int best = 8;
     double fill = 0.0;
     for (int b = 8; b >= 5; --b) {
