@@ -160,11 +160,24 @@ __device__ __forceinline__ void put(f32x2 (&a)[CM], int c, f32x2 v) {
         if (k == c) a[k] = v;
 }
 
-// Mean counts yb[c] = sum_E S t of both rays.
-template <int NM, int CM>
-__device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], f32x2 (&yb)[CM]) {
+// Mean counts yb[c] = sum_E S t of both rays; with TOP also the largest exponent
+// of 2 met over all energies (-log2(e) times the smallest z), from the same
+// pass.
+template <bool TOP, int NM, int CM>
+__device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], f32x2 (&yb)[CM], float &za,
+                                        float &zb) {
 #pragma unroll
     for (int c = 0; c < CM; ++c) yb[c] = 0ull;
+    za = zb = -3.0e38f;
+    auto exponent = [&](const f32x2 (&q)[NM]) {
+        const f32x2 z = neglog2e(dot2(q, l));
+        if constexpr (TOP) {
+            float a, b;
+            unpair2(z, a, b);
+            za = fmaxf(za, a), zb = fmaxf(zb, b);
+        }
+        return z;
+    };
     for_segments(
         tab,
         [&](int c, int e0, int e1) {
@@ -173,7 +186,7 @@ __device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s;
                 tab.get(e, c, q, s);
-                a = fma2(s, exp2_pair(neglog2e(dot2(q, l))), a);
+                a = fma2(s, exp2_pair(exponent(q)), a);
             }
             put(yb, c, a);
         },
@@ -182,12 +195,26 @@ __device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 
             for (int e = e0; e < e1; ++e) {
                 f32x2 q[NM], s[CM];
                 tab.get(e, q, s);
-                const f32x2 t = exp2_pair(neglog2e(dot2(q, l)));
+                const f32x2 t = exp2_pair(exponent(q));
 #pragma unroll
                 for (int c = 0; c < CM; ++c) yb[c] = fma2(s[c], t, yb[c]);
             }
         },
-        [](int, int) {});
+        [&](int e0, int e1) {
+            if constexpr (TOP) {
+                for (int e = e0; e < e1; ++e) {
+                    f32x2 q[NM], s;
+                    tab.get(e, 0, q, s);
+                    exponent(q);
+                }
+            }
+        });
+}
+
+template <int NM, int CM>
+__device__ __forceinline__ void counts2(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], f32x2 (&yb)[CM]) {
+    float za, zb;
+    counts2<false>(tab, l, yb, za, zb);
 }
 
 // Gradient numerators gm = -sum_E Q t v, v = -sum_c S u_c (u the negated weighted
@@ -365,19 +392,6 @@ struct SegPair {
         p[t[1]] = valid[1] ? b : 0.f;
     }
 };
-
-// Largest exponent of 2 met over all energies.
-template <int NM, int CM>
-__device__ __forceinline__ void top_exponent(const SpecTab<NM, CM> &tab, const f32x2 (&l)[NM], float &za, float &zb) {
-    za = zb = -3.0e38f;
-    for (int e = 0; e < tab.ne; ++e) {
-        f32x2 q[NM], s;
-        tab.get(e, 0, q, s);
-        float a, b;
-        unpair2(neglog2e(dot2(q, l)), a, b);
-        za = fmaxf(za, a), zb = fmaxf(zb, b);
-    }
-}
 
 template <int NM, int CM, bool KAPPA>
 __global__ void __launch_bounds__(kModelThreads)
@@ -853,10 +867,8 @@ __global__ void __launch_bounds__(kModelThreads)
 #pragma unroll
                     for (int m = 0; m < NM; ++m) nq[m] = sub2(0ull, qm[m]);
                     line2(tab, la, nq, v0, v1, v2, ze[0], ze[1]);
-                }
-                else {
-                    counts2(tab, la, v0);
-                    top_exponent(tab, la, ze[0], ze[1]);
+                } else {
+                    counts2<true>(tab, la, v0, ze[0], ze[1]);
                 }
 #pragma unroll
                 for (int c = 0; c < CM; ++c)
