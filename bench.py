@@ -47,16 +47,15 @@ DEVLS_BYTES = 80
 # workload (summaries under profiles/): DRAM bytes read + written per launch,
 # and the unit that binds it.  Remove an entry when its kernel changes.
 NCU_CAPTURES = {
-    # 128^3 capture of the same kernel (back_cols_kernel<4, 4>), 148.3 MB per
-    # launch, scaled by the rays and voxels processed (8x each) to 256^3
+    # DRAM bytes of one launch at 256^3; the binding unit from the 128^3 capture
     ("c5_cone3d_256_block", "backproject"): {
-        "traffic": 8 * 148.3e6,
-        "binding": {"unit": "L1 / shared-memory throughput (% of peak)", "frac_of_peak": 0.631,
-                    "source": "profiles/back_cols_c5_128.md"},
+        "traffic": 2.325e9,
+        "binding": {"unit": "L1 / shared-memory throughput (% of peak)", "frac_of_peak": 0.625,
+                    "source": "profiles/back_cols_c5_128.md, profiles/launches_c5_cone256_block.md"},
     },
     ("c2_fan2d_512_haar", "backproject"): {
         "traffic": 16.13e6,
-        "binding": {"unit": "SM instruction issue (issue active, % of cycles)", "frac_of_peak": 0.833,
+        "binding": {"unit": "SM instruction issue (issue active, % of cycles)", "frac_of_peak": 0.834,
                     "source": "profiles/back_tile_2d_c2_fan512.md"},
     },
 }

@@ -36,14 +36,13 @@ __device__ __forceinline__ float transmission(float z) { return exp2f(z * -1.442
 // line integrals (two materials: 3.30e-7 instead of 3.17e-7, since a rounded
 // line integral errs alike at every energy) saves that, 3 % of a
 // projection-domain iteration.
-// Measured on 720 x 888 rays, 2 materials, 121 energies, 2 channels (ncu, cold):
-// numerators 117 -> 80 us, line-search evaluation 76 -> 55 us, the eight halving
-// candidates 181 -> 107 us against one ray per thread with exp2f's subnormal
-// handling and every channel at every energy; 3 materials, 4 channels: model
-// stage 146 -> 85 us, line search 395 -> 231 us per iteration; with blur and
-// correlated noise the data-term gradient 174 -> 96 us.  The FP32 pipe is half
-// busy and so is issue (50 % each for the evaluation); more rays (x 8) run at
-// the same rate.
+// Measured on 720 x 888 rays, 2 materials, 121 energies, 2 channels, against one
+// ray per thread with exp2f's subnormal handling and every channel at every
+// energy: numerators 117 -> 84 us, line-search evaluation 76 -> 57 us (ncu, cold);
+// 3 materials, 4 channels: model stage 148 -> 89 us, line search 508 -> 322 us per
+// iteration, halvings included; with blur and correlated noise the data-term
+// gradient 175 -> 100 us.  The FP32 pipe and issue are half busy (54 % and 52 %
+// for the evaluation); more rays (x 8) run at the same rate.
 constexpr float kLog2e = 1.4426950408889634f;
 
 // Exponents of 2 that give exp(-z).
